@@ -203,6 +203,7 @@ struct InstDev {
     size_t o_Qsym = 0;    // symmetric storage tiles
     size_t o_Uhi, o_Ulo;
     size_t o_spv = 0, o_spc = 0, o_spo = 0;   // sliced storage (in the second allocation)
+    int max_width = 0;                        // sliced storage: entries of the longest row
     int bn, n_tiles, rows_b;   // tensor-core tiling of this instance's lanes
     int lane0, nl;
 };
@@ -396,6 +397,8 @@ class Solver {
         o_active_ = ar_.reserve(sizeof(int32_t));
         o_bytes_ = ar_.reserve(sizeof(unsigned long long));
 
+        lane_inst_.resize(lanes.size());
+        for (size_t l = 0; l < lanes.size(); ++l) lane_inst_[l] = lanes[l].inst;
         // lanes: rows per phase-A item for the GEMV path
         int64_t total_rows = 0;
         for (const LaneIn& l : lanes) total_rows += insts[l.inst].n;
@@ -470,12 +473,12 @@ class Solver {
         o_p0_.assign(lanes.size(), SIZE_MAX);
         sym_host_.assign(sym_ ? lanes.size() : 0, SymLane());
         o_pbuf_.assign(lanes.size(), 0);
+        std::vector<size_t> xch(lanes.size(), 0);   // exchange words of sliced lanes on CTA groups
+        size_t xch_words = 0;
         int64_t nitems = 0;
-        lane_inst_.assign(lanes.size(), 0);
         for (size_t l = 0; l < lanes.size(); ++l) {
             const LaneIn& in = lanes[l];
             InstDev& I = inst_[in.inst];
-            lane_inst_[l] = in.inst;
             if (I.lane0 < 0) I.lane0 = (int)l;
             I.nl += 1;
             LaneDev& L = lanes_[l];
@@ -498,6 +501,8 @@ class Solver {
             o_bx_[l] = ar_.reserve((size_t)I.ld);
             // the single-lane kernel's one-barrier steps alternate between two sets of records
             o_part_[l] = ar_.reserve((size_t)(solo_ ? 2 : 1) * L.nblk * sizeof(Partial));
+            xch[l] = xch_words;
+            if (solo_ && sparse_) xch_words += (size_t)kSellWordsPerBlock * L.nblk;
             if (in.trace_len > 0) {
                 o_trace_x_[l] = ar_.reserve((size_t)in.trace_len * I.n * 4);
                 o_trace_a_[l] = ar_.reserve((size_t)in.trace_len * 4);
@@ -526,6 +531,7 @@ class Solver {
         o_symctr_ = sym_ ? ar_.reserve(lanes.size() * sizeof(unsigned int)) : 0;
         o_symlanes_ = sym_ ? ar_.reserve(lanes.size() * sizeof(SymLane)) : 0;
         o_queue_ = ar_.reserve(2 * sizeof(int32_t));
+        const size_t o_xch = ar_.reserve(xch_words * sizeof(ulonglong2));
         // single-lane kernel: err, active_after, then one barrier of kSoloBarStride words per group,
         // then the group tables
         // (room for the largest plan: a group per lane, or one per resident CTA)
@@ -584,6 +590,8 @@ class Solver {
         UBQP_CK(cudaMemsetAsync(ar_.at<char>(o_queue_), 0, 2 * sizeof(int32_t), stream_));
         UBQP_CK(cudaMemsetAsync(ar_.at<char>(o_solo_), 0, (4 + nsg * kSoloBarStride) * sizeof(int32_t), stream_));
         if (solo_) UBQP_CK(upload_solo_plan());
+        // no exchange word carries a step's tag yet
+        if (xch_words > 0) UBQP_CK(cudaMemsetAsync(ar_.at<char>(o_xch), 0, xch_words * sizeof(ulonglong2), stream_));
         UBQP_CK(cudaMemsetAsync(ar_.at<char>(o_valid_), 0, insts.size() * 4 * sizeof(float), stream_));
         UBQP_CK(cudaMemsetAsync(ar_.at<char>(o_nnz_), 0, insts.size() * sizeof(unsigned long long), stream_));
         UBQP_CK(cudaMemsetAsync(ar_.at<char>(o_scal_), 0, insts.size() * 4 * sizeof(float), stream_));
@@ -747,6 +755,7 @@ class Solver {
                 L.spc = sp_ar_.at<uint16_t>(I.o_spc);
                 L.spo = sp_ar_.at<int64_t>(I.o_spo);
                 L.spwps = 256 / rows_per_item_;   // 256 threads per GEMV CTA
+                L.xch = solo_ ? ar_.at<ulonglong2>(o_xch) + xch[l] : nullptr;
             }
             L.Qeval = tc ? nullptr : ar_.at<float2>(I.o_Qeval);
             L.d = ar_.at<float>(I.o_d);
@@ -1223,6 +1232,7 @@ class Solver {
             I.o_spv = sp_ar_.reserve(std::max<size_t>(entries, 1) * 4);
             I.o_spc = sp_ar_.reserve(std::max<size_t>(entries, 1) * 2);
             I.o_spo = sp_ar_.reserve((ns + 1) * 8);
+            I.max_width = ns ? *std::max_element(w.begin() + sl0[t], w.begin() + sl0[t] + ns) : 0;
             sliced_entries_ += (int64_t)entries;
         }
         int rc = sp_ar_.commit();
@@ -1254,7 +1264,13 @@ class Solver {
             sa.gfirst = tab + solo_nl_;
             sa.gcta = sa.gfirst + solo_gmax_ + 1;
             sa.grid = solo_gcta_.back();
+            sell_ = sell_shape(&sell_smem_, &sa.mat_bytes);
         };
+        if (nlanes_ > 1 && sparse_) {   // the widths are known now: the plan whose slices fit best
+            std::vector<int> ids(nlanes_);
+            for (int l = 0; l < nlanes_; ++l) ids[l] = l;
+            if (plan_solo_groups(ids, max_ld_, true)) UBQP_CK(upload_solo_plan());
+        }
         set_plan();
         sa.rows_per_item = rows_per_item_;
         sa.budget = probe_ticks_ > 0 ? probe_ticks_ : (o_.lane_budget > 0 ? o_.lane_budget : 1024);
@@ -1263,6 +1279,8 @@ class Solver {
         sa.active_after = ctl + 1;
         sa.bar = reinterpret_cast<unsigned*>(ctl + 4);
         sa.wait_ns = o_.wait_limit_us > 0 ? 1000ull * (unsigned long long)o_.wait_limit_us : 5000000000ull;
+        // (the highest SM clock is 2070 MHz; asking the runtime for it takes 600 us)
+        sa.wait_cycles = sa.wait_ns / 1000ull * 2100ull;
         sa.fast = 1;
         sa.one_ok = solo_one_ok_ ? 1 : 0;
         sa.P = make_params(o_, ar_.at<int64_t>(o_hist_));
@@ -1282,7 +1300,8 @@ class Solver {
         for (;;) {
             UBQP_CK(cudaMemsetAsync(sa.active_after, 0, sizeof(int32_t), stream_));
             if (prof) UBQP_CK(cudaEventRecord(evA_[0], stream_));
-            UBQP_CK(launch_solo(sa, max_ld_, stream_));
+            if (sell_) UBQP_CK(launch_sell(sa, solo_per_, sell_smem_, stream_));
+            else UBQP_CK(launch_solo(sa, max_ld_, stream_));
             if (prof) UBQP_CK(cudaEventRecord(evA_[1], stream_));
             UBQP_CK(cudaMemcpyAsync(h_active_, ctl, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, stream_));
             launches_ += 1;
@@ -1359,14 +1378,28 @@ class Solver {
         int max_lanes = 1;
         int maxnb = 0;
         for (int l : ids) maxnb = std::max(maxnb, solo_nb_[l]);
+        solo_per_ = (int)(capc / num_sms_);
         if ((int64_t)nl <= capc) {
-            int m = 1;
-            for (; m <= maxnb; ++m) {
-                int64_t tot = 0;
-                for (int l : ids) tot += (solo_nb_[l] + m - 1) / m;
-                if (tot <= capc) break;
+            int m = 0;
+            double best = INFINITY;
+            // fewer, larger CTAs (per SM) or more, smaller ones: the smallest m of each, and of
+            // these the one with the least work per SM and step
+            for (int per = 1; per <= 2 && per * num_sms_ <= capc; ++per) {
+                int mp = 1;
+                for (; mp <= maxnb; ++mp) {
+                    int64_t tot = 0;
+                    for (int l : ids) tot += (solo_nb_[l] + mp - 1) / mp;
+                    if (tot <= (int64_t)per * num_sms_) break;
+                }
+                if (mp > maxnb || (!forced && mp > kSoloMaxSl)) continue;
+                const double c = solo_cost(ids, per, mp, max_ld);
+                if (c < best) {
+                    best = c;
+                    m = mp;
+                    solo_per_ = per;
+                }
             }
-            if (!forced && m > kSoloMaxSl) return false;
+            if (m == 0) return false;
             for (int l : order) {
                 gl.push_back(l);
                 gf.push_back((int)gl.size());
@@ -1394,6 +1427,42 @@ class Solver {
         solo_gcta_ = gc;
         solo_max_lanes_ = std::max(solo_max_lanes_, max_lanes);
         return true;
+    }
+
+    // Relative cost of a step with `per` CTAs of m slices on an SM: a slice whose entries stay in
+    // shared memory costs its gathers there, about 3.5 cycles per entry and warp (32 lanes meet
+    // in about as many banks), a slice read from L2 five times that (latency)
+    double solo_cost(const std::vector<int>& ids, int per, int m, int max_ld) const
+    {
+        int w = 0;
+        for (int l : ids) w = std::max(w, inst_[(size_t)lane_inst_[l]].max_width);
+        if (m > kSoloMaxSl || w == 0 || rows_per_item_ != 32) return 1e9 + 1e3 * m + per;   // solo.cu: the smallest m
+        const int64_t room = (int64_t)sell_smem_limit(per) - 2 * (int64_t)max_ld * (int64_t)sizeof(float);
+        const int64_t res = std::max<int64_t>(0, std::min<int64_t>(m, room / (192 * (int64_t)w)));
+        return per * w * (3.5 * (double)res + 17.5 * (double)(m - res));
+    }
+
+    // Whether the current plan runs on the sliced kernel (sell_lane.cu), and its shared memory:
+    // two vectors and as many of a CTA's slices as fit
+    bool sell_shape(size_t* smem, int32_t* mat_bytes) const
+    {
+        if (!sparse_) return false;
+        size_t mat = 0;
+        for (size_t g = 0; g + 1 < solo_gcta_.size(); ++g)
+            for (int q = solo_gfirst_[g]; q < solo_gfirst_[g + 1]; ++q) {
+                const LaneDev& L = lanes_[(size_t)solo_glanes_[q]];
+                const int nc = solo_gcta_[g + 1] - solo_gcta_[g];
+                const bool one = nc == 1 && L.nblk == 1;
+                if (!one && (rows_per_item_ != 32 || (L.nblk + nc - 1) / nc > kSoloMaxSl)) return false;
+                const size_t slices = one ? (size_t)(L.n + 31) / 32 : (size_t)((L.nblk + nc - 1) / nc);
+                mat = std::max(mat, slices * (size_t)inst_[(size_t)lane_inst_[solo_glanes_[q]]].max_width * 192);
+            }
+        const size_t limit = sell_smem_limit(solo_per_), vecs = 2 * (size_t)max_ld_ * sizeof(float);
+        if (vecs > limit) return false;
+        mat = std::min(mat, limit - vecs);
+        *smem = vecs + mat;
+        *mat_bytes = (int32_t)mat;
+        return solo_per_ <= 2 && sell_fits(solo_per_, *smem);
     }
 
     // the group tables to the device (glanes, then gfirst and gcta at fixed offsets) and the
@@ -1694,6 +1763,9 @@ class Solver {
     bool solo_one_ok_ = false;
     int solo_max_lanes_ = 1;
     int64_t solo_capc_ = 0;      // CTAs resident at once
+    int solo_per_ = 1;           // CTAs of the current plan that share an SM
+    bool sell_ = false;          // the current plan runs on the sliced kernel
+    size_t sell_smem_ = 0;
     size_t solo_gmax_ = 1;       // groups the tables and barriers have room for
     int solo_nl_ = 0;            // lanes (the tables' first part)
     int loop_grid_ = 0, loop_budget_ = 0;

@@ -227,6 +227,35 @@ static __host__ __device__ __noinline__ bool rayleigh_ritz(const float (&ga)[6],
 
 __device__ __forceinline__ float csum_value(float2 v) { return v.x + v.y; }
 
+// The scalar step of one inner iteration k from its reduced sums (ss = s^T s, sy = s^T y, yy = y^T y)
+// and maxima: rho of Eq. (cret) and the first step at k = 0, the KKT test, and for Alg. 2 the
+// alternating BB step of Eq. (bb1) with its safeguards.  Returns the subproblem's exit code or
+// -1 to step on; alpha is the step to take.
+__device__ __forceinline__ int inner_scalar(int method, int k, int max_inner, float tol, float alpha_min, float alpha_max,
+                                            float qmax_off, const float* m, float ss, float sy, float yy, float& rho,
+                                            float& alpha)
+{
+    if (k == 0) {
+        rho = fmaxf(fmaxf(1.f, 2.f * qmax_off), fmaxf(2.f * m[1], m[2]));
+        alpha = m[3] > 0.f ? 1.f / (2.f * m[3]) : 1.f;
+    }
+    // the two quotients side by side (they are most of the step's latency)
+    const bool odd = k & 1;
+    const float viol = m[0] / rho;
+    float a = (odd ? ss : sy) / (odd ? sy : yy);
+    if (viol < tol) return 0;
+    if (k >= max_inner) return 1;
+    if (k < 1) return -1;
+    // Alg. 1 ends when the projected step left x unchanged (s = x_k - x_{k-1} = 0): in FP32 a
+    // step g / (2 h_p) below half an ulp of x stalls the iteration; so does Alg. 2
+    if (ss == 0.f) return 2;
+    if (method == 0) {
+        if (!(sy > 0.f) || !isfinite(a)) a = alpha;
+        alpha = fminf(fmaxf(a, alpha_min), alpha_max);
+    }
+    return -1;
+}
+
 // Scalar decision of one lane (thread 0).  S is the lane state (shared memory).
 static __device__ void decide(const LaneDev& L, LaneState& S, const Partial& R, const Params& P, Decision& D)
 {
@@ -344,27 +373,8 @@ static __device__ void decide(const LaneDev& L, LaneState& S, const Partial& R, 
     case PH_INNER: {
         S.inner_iters += 1;
         const int k = S.k;
-        if (k == 0) {
-            S.rho = fmaxf(fmaxf(1.f, 2.f * L.qmax_off), fmaxf(2.f * R.m[1], R.m[2]));
-            S.alpha = R.m[3] > 0.f ? 1.f / (2.f * R.m[3]) : 1.f;
-        }
-        int exit_code = -1;
-        if (R.m[0] / S.rho < P.tol_inner) exit_code = 0;
-        else if (k >= P.max_inner) exit_code = 1;
-        else if (L.method == 1 && k >= 1) {
-            // Alg. 1 ends when the projected step left x unchanged (s = x_k - x_{k-1} = 0): in
-            // FP32 a step g / (2 h_p) below half an ulp of x stalls the iteration
-            if (csum_value(R.s[0]) == 0.f) exit_code = 2;
-        } else if (L.method == 0 && k >= 1) {
-            float ss = csum_value(R.s[0]), sy = csum_value(R.s[1]), yy = csum_value(R.s[2]);
-            if (ss == 0.f) exit_code = 2;
-            else {
-                float a = (k & 1) ? ss / sy : sy / yy;
-                if (!(sy > 0.f) || !isfinite(a)) a = S.alpha;
-                a = fminf(fmaxf(a, P.alpha_min), P.alpha_max);
-                S.alpha = a;
-            }
-        }
+        const int exit_code = inner_scalar(L.method, k, P.max_inner, P.tol_inner, P.alpha_min, P.alpha_max, L.qmax_off, R.m,
+                                           csum_value(R.s[0]), csum_value(R.s[1]), csum_value(R.s[2]), S.rho, S.alpha);
         if (L.trace_len > 0 && k < L.trace_len && exit_code < 0) {
             D.act |= A_TRACE;
             D.trace_k = k;

@@ -19,9 +19,9 @@
 // it.  g alternates between two global buffers by the parity of k (V_G, V_W), and so do the
 // blocks' partial records (the lane holds two sets), so a CTA that has passed the step's barrier
 // and computes step k+1 never overwrites g_k or a record of step k that another CTA of the
-// group may still be reading.  On the sliced storage with one slice per block, a CTA computes
-// its slices one after another, each with sixteen entries per thread in flight.  When the subproblem ends,
-// or the launch's budget does, the CTAs write x_k, x_{k-1} and u back.  The arithmetic is that
+// group may still be reading.  When the subproblem ends, or the launch's budget does, the CTAs write x_k,
+// x_{k-1} and u back.  Lanes on the sliced storage run sell_lane.cu instead, except those whose
+// blocks are not 32 rows or whose CTAs own more than kSoloMaxSl slices.  The arithmetic is that
 // of the lock-step scheduler with the same rows per item, so both give the same bits.  Every
 // group barrier wait is bounded: when it runs out the CTA sets the error flag and leaves, and
 // the others leave at their own next wait.  A group of one CTA needs no barrier.
@@ -29,83 +29,9 @@
 // Lane vectors and partial records written by one CTA are read by others within the launch,
 // so this file is compiled with plain loads cached in L2 only (-dlcm=cg); Q keeps its
 // non-coherent streaming loads.
-#include "gemv_rows.cuh"
+#include "solo_common.cuh"
 
 namespace ubqp {
-
-__device__ __forceinline__ uint64_t solo_clock()
-{
-    uint64_t t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-
-__device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long* p)
-{
-    unsigned long long v;
-    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
-
-// Group barrier on a monotonic 64-bit arrival counter: barrier number gen + 1 of the group is
-// complete when the counter reaches nc * (gen + 1).  A CTA adds its arrival without waiting for
-// the result and polls the counter (bounded); nobody resets anything, so a barrier costs one
-// round trip after the last arrival.
-__device__ __forceinline__ bool solo_grid_sync(const SoloArgs& A, unsigned long long* bar, int nc,
-                                               unsigned long long& gen, int* s_ok)
-{
-    __syncthreads();
-    if (nc == 1) return *s_ok != 0;
-    if (threadIdx.x == 0) {
-        const unsigned long long target = (gen + 1ull) * (unsigned long long)nc;
-        __threadfence();
-        asm volatile("red.relaxed.gpu.global.add.u64 [%0], 1;" ::"l"(bar) : "memory");
-        const uint64_t t0 = solo_clock();
-        while (ld_acquire_u64(bar) < target) {
-            if (solo_clock() - t0 > A.wait_ns) {
-                atomicExch(A.err, 1);
-                *s_ok = 0;
-                break;
-            }
-        }
-        gen += 1ull;
-    }
-    __syncthreads();
-    return *s_ok != 0;
-}
-
-// Alg. 2 row epilogue of the single-barrier step for row i: x_k, x_{k-1}, d - p, d + b' and
-// g_{k-1} of the row given, g_k written to gnew[i] and returned; the arithmetic of row_epilogue
-// (PH_INNER)
-__device__ __forceinline__ float solo_inner_row(const LaneDev& L, int k, int i, float v, float x, float xp, float dmp,
-                                                float tsum, float gold, float* gnew, Acc& a)
-{
-    const float g = fmaf(dmp, 2.f * x - 1.f, fmaf(2.f, v, tsum));
-    if (k >= 1) {
-        const float sd = x - xp;
-        const float y = g - gold;
-        csum_add(a.s[0], sd * sd);
-        csum_add(a.s[1], sd * y);
-        csum_add(a.s[2], y * y);
-    } else {
-        a.m[1] = fmaxf(a.m[1], fabsf(dmp));
-        a.m[2] = fmaxf(a.m[2], fabsf(L.vec[V_BBAR * L.ld + i]));
-        a.m[3] = fmaxf(a.m[3], L.oabs[i] + fabsf(dmp));
-    }
-    gnew[i] = g;
-    const float viol = (x > 0.f && x < 1.f) ? fabsf(g) : (x <= 0.f ? fmaxf(-g, 0.f) : fmaxf(g, 0.f));
-    a.m[0] = fmaxf(a.m[0], viol);
-    return g;
-}
-
-__device__ __forceinline__ unsigned long long solo_item_bytes(const LaneDev& L, int blk, int row0, int rows)
-{
-    if (L.spv)
-        return 6ull * (unsigned long long)(L.spo[(row0 + rows + 31) >> 5] - L.spo[row0 >> 5]) +
-               (blk == 0 ? 4ull * L.n : 0ull) + 16ull * rows;
-    return (unsigned long long)rows * L.n * 4ull + (blk == 0 ? 4ull * L.n : 0ull) + 16ull * rows;
-}
 
 // the row epilogue of one block and its partial record, by the whole CTA
 __device__ __forceinline__ void solo_inner_finish(const LaneDev& L, int k, int blk, int row0, int rows,
@@ -121,100 +47,6 @@ __device__ __forceinline__ void solo_inner_finish(const LaneDev& L, int k, int b
     }
     block_reduce_write<kWarps>(a, PH_INNER, out, false);
     if (P.bytes && threadIdx.x == 0) atomicAdd(P.bytes, solo_item_bytes(L, blk, row0, rows));
-}
-
-// The same epilogue and record for a block of at most 32 rows, by one warp (lane r: row r).
-// block_reduce_write over the CTA would merge this warp's sums with seven warps' zero sums in
-// warp order; the merges below are those, so the record has the same bits.
-__device__ __forceinline__ void solo_inner_finish_warp(const LaneDev& L, int k, int blk, int row0, int rows,
-                                                       const double* sv, const Params& P, const float* sx,
-                                                       const float* sxp, float* gnew, float dmp, float tsum,
-                                                       float gold, Partial* out, int lane)
-{
-    Acc a;
-    a.zero();
-    if (lane < rows) {
-        const int i = row0 + lane;
-        solo_inner_row(L, k, i, (float)sv[lane], sx[i], sxp[i], dmp, tsum, gold, gnew, a);
-    }
-#pragma unroll
-    for (int t = 0; t < 3; ++t) a.s[t] = csum_shfl_reduce(a.s[t]);
-#pragma unroll
-    for (int t = 0; t < 4; ++t) a.m[t] = max_shfl_reduce(a.m[t]);
-    if (lane == 0) {
-        Partial R;
-        const float2 z2 = make_float2(0.f, 0.f);
-        for (int t = 0; t < 12; ++t) R.s[t] = z2;
-        for (int t = 0; t < 6; ++t) R.m[t] = 0.f;
-        R.f = 0.0;
-        const int ns = phase_nsum(PH_INNER), nm = phase_nmax(PH_INNER);
-        for (int t = 0; t < ns; ++t) R.s[t] = csum_merge(R.s[t], a.s[t]);
-        for (int t = 0; t < nm; ++t) R.m[t] = fmaxf(R.m[t], a.m[t]);
-        R.f += 0.0;
-        for (int w = 1; w < kWarps; ++w) {
-            for (int t = 0; t < ns; ++t) R.s[t] = csum_merge(R.s[t], z2);
-            for (int t = 0; t < nm; ++t) R.m[t] = fmaxf(R.m[t], 0.f);
-            R.f += 0.0;
-        }
-        *out = R;
-        if (P.bytes) atomicAdd(P.bytes, solo_item_bytes(L, blk, row0, rows));
-    }
-}
-
-// Products of one 32-row slice (sliced storage) for sv[r]: the shares, operations and merge of
-// item_rows_sell with eight warps per slice, the loads sixteen entries of the share at a time
-// (a CTA with a single slice waits for fewer load rounds)
-__device__ __forceinline__ void solo_rows_one(const LaneDev& L, int sl, int rows, const float* su, double* sv,
-                                              float2* s_share1, int lane, int warp)
-{
-    const int64_t base = L.spo[sl];
-    const int width = (int)((L.spo[sl + 1] - base) >> 5);
-    const int k0 = width * warp / kWarps, k1 = width * (warp + 1) / kWarps;
-    const float* V = L.spv + base + lane + 32 * (int64_t)k0;
-    const uint16_t* C = L.spc + base + lane + 32 * (int64_t)k0;
-    const int ng = ((k1 - k0) >> 3) * 2;   // groups of four summed as FMA groups
-    float2 acc = make_float2(0.f, 0.f);
-    int j = 0;
-    for (; j + 4 <= ng; j += 4) {
-        float q[16];
-        int c[16];
-#pragma unroll
-        for (int e = 0; e < 16; ++e) {
-            q[e] = __ldg(V + 32 * (4 * j + e));
-            c[e] = __ldg(C + 32 * (4 * j + e));
-        }
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-            float t = __fmul_rn(q[4 * h], su[c[4 * h]]);
-            t = fmaf(q[4 * h + 1], su[c[4 * h + 1]], t);
-            t = fmaf(q[4 * h + 2], su[c[4 * h + 2]], t);
-            t = fmaf(q[4 * h + 3], su[c[4 * h + 3]], t);
-            csum_add(acc, t);
-        }
-    }
-    for (; j < ng; ++j) {
-        float q[4];
-        int c[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            q[e] = __ldg(V + 32 * (4 * j + e));
-            c[e] = __ldg(C + 32 * (4 * j + e));
-        }
-        float t = __fmul_rn(q[0], su[c[0]]);
-        t = fmaf(q[1], su[c[1]], t);
-        t = fmaf(q[2], su[c[2]], t);
-        t = fmaf(q[3], su[c[3]], t);
-        csum_add(acc, t);
-    }
-    for (int k = 4 * ng; k < k1 - k0; ++k) csum_add(acc, __fmul_rn(__ldg(V + 32 * k), su[__ldg(C + 32 * k)]));
-    s_share1[lane * kWarps + warp] = acc;
-    __syncthreads();
-    if ((int)threadIdx.x < rows) {
-        const float2* sh = s_share1 + threadIdx.x * kWarps;
-        float2 a = sh[0];
-        for (int w = 1; w < kWarps; ++w) a = csum_merge(a, sh[w]);
-        sv[threadIdx.x] = (double)(a.x + a.y);
-    }
 }
 
 // x_{k+1} = P(x_k - alpha g_k) over the whole padded vector (ld a multiple of 4), g_k from global
@@ -256,7 +88,6 @@ __global__ void __launch_bounds__(kThreads, 2) solo_lane_kernel(SoloArgs A)
     __shared__ Decision D;
     __shared__ int s_ok, s_g;
     __shared__ unsigned long long s_gen0;
-    __shared__ float2 s_share[kSoloMaxSl][kThreads];
     __shared__ Partial s_part;
     // the descriptor never changes: one copy in shared memory (this file's plain loads go to
     // L2, so every field read from global memory would be an L2 round trip)
@@ -345,17 +176,6 @@ __global__ void __launch_bounds__(kThreads, 2) solo_lane_kernel(SoloArgs A)
             tsumv = stsum;
             __syncthreads();
         }
-        // this CTA's blocks (sliced storage, 32 rows per item: all of them before one barrier)
-        const bool multi = L.spv && A.rows_per_item == 32 && (nblk + nc - 1) / nc <= kSoloMaxSl;
-        int my_sl[kSoloMaxSl];
-        int my_n = 0;
-#pragma unroll
-        for (int b = 0; b < kSoloMaxSl; ++b) {
-            const int blk = rank + b * nc;
-            my_sl[b] = blk;
-            if (blk < nblk) my_n = b + 1;
-        }
-
         for (; steps_left > 0; --steps_left) {
             const int ph = S.phase;
             if (ph == PH_DONE) break;
@@ -373,41 +193,16 @@ __global__ void __launch_bounds__(kThreads, 2) solo_lane_kernel(SoloArgs A)
                 __syncthreads();
             }
             // ---- phase A: this CTA's row block(s)
-            if (fast_step && multi) {
-                if (my_n > 0) {
-                    // the epilogue's per-row operands of warp w's block (d - p, d + b', g_{k-1}),
-                    // loaded before the products so that their round trip overlaps them
-                    float e_dmp = 0.f, e_ts = 0.f, e_g = 0.f;
-                    if (warp < my_n) {
-                        const int i = min(my_sl[warp] * 32 + lane, L.n - 1);
-                        e_dmp = dmpv[i];
-                        e_ts = tsumv[i];
-                        if (k >= 1) e_g = gbuf[(k + 1) & 1][i];
-                    }
-                    // the CTA's slices one after another, each into its own share buffer (measured
-                    // faster than interleaving the slices' loads, which cost registers)
-                    for (int b = 0; b < my_n; ++b)
-                        solo_rows_one(L, my_sl[b], min(32, L.n - my_sl[b] * 32), su, sv + 32 * b, s_share[b], lane, warp);
-                    __syncthreads();
-                    if (warp < my_n) {
-                        const int blk = my_sl[warp], row0 = blk * 32;
-                        solo_inner_finish_warp(L, k, blk, row0, min(32, L.n - row0), sv + 32 * warp, P, su, sxp,
-                                               gbuf[k & 1], e_dmp, e_ts, e_g,
-                                               one ? &s_part : L.part + (size_t)(k & 1) * nblk + blk, lane);
-                    }
-                }
-            } else {
-                for (int blk = rank; blk < nblk; blk += nc) {
-                    const int row0 = blk * A.rows_per_item;
-                    const int rows = min(A.rows_per_item, L.n - row0);
-                    item_rows_solver(L, ph, row0, rows, su, sv, lane, warp);
-                    __syncthreads();
-                    if (fast_step)
-                        solo_inner_finish(L, k, blk, row0, rows, sv, P, su, sxp, gbuf[(k + 1) & 1], gbuf[k & 1], dmpv,
-                                          tsumv, one ? &s_part : L.part + (size_t)(k & 1) * nblk + blk);
-                    else item_finish(L, ph, k, blk, row0, rows, sv, P);
-                    __syncthreads();
-                }
+            for (int blk = rank; blk < nblk; blk += nc) {
+                const int row0 = blk * A.rows_per_item;
+                const int rows = min(A.rows_per_item, L.n - row0);
+                item_rows_solver(L, ph, row0, rows, su, sv, lane, warp);
+                __syncthreads();
+                if (fast_step)
+                    solo_inner_finish(L, k, blk, row0, rows, sv, P, su, sxp, gbuf[(k + 1) & 1], gbuf[k & 1], dmpv, tsumv,
+                                      one ? &s_part : L.part + (size_t)(k & 1) * nblk + blk);
+                else item_finish(L, ph, k, blk, row0, rows, sv, P);
+                __syncthreads();
             }
             if (!solo_grid_sync(A, bar, nc, gen, &s_ok)) break;
             // ---- the update: the same reduction and decision in every CTA (one CTA in Alg. 2: its

@@ -135,6 +135,8 @@ struct LaneDev {
     const float* spv;
     const uint16_t* spc;
     const int64_t* spo;
+    ulonglong2* xch;       // sliced lanes on groups of CTAs: the exchange words (kSellWordsPerBlock
+                           // per row block, zeroed before the first launch), else null
 };
 
 // solver constants (kernel parameter)
@@ -500,9 +502,13 @@ struct SoloArgs {
     unsigned* bar;              // per group (stride kSoloBarStride words): a 64-bit arrival counter
     int32_t* err;               // set when a bounded wait runs out
     int32_t* active_after;      // lanes unfinished at the end of the launch (the caller zeroes it)
-    unsigned long long wait_ns; // limit of one barrier wait
+    unsigned long long wait_ns; // limit of one wait of a CTA for the others of its group ...
+    unsigned long long wait_cycles;   // ... in SM cycles (at the highest SM clock, so never shorter);
+                                // the waits read the SM's own counter: reading the global timer
+                                // takes longer than the wait it would bound
     int32_t fast;               // Alg. 2 steps with one barrier (whole x_k in every CTA)
     int32_t one_ok;             // shared memory holds the one-CTA state (6 vectors)
+    int32_t mat_bytes;          // sell_lane.cu: shared memory of a CTA for its slices' entries
     Params P;
 };
 constexpr int kSoloBarStride = 32;   // unsigned per group barrier (128 bytes)
@@ -512,6 +518,13 @@ size_t solo_smem(int ld, bool one);
 cudaError_t prepare_solo(int ld, bool one);
 int solo_ctas_per_sm(int ld, bool one);
 cudaError_t launch_solo(const SoloArgs& a, int ld, cudaStream_t s);
+
+// the same groups on the sliced storage, at most kSoloMaxSl slices per CTA (or a lane of one block
+// on one CTA): entries in shared memory, one-hop exchanges (sell_lane.cu)
+constexpr int kSellWordsPerBlock = 74;   // 16-byte exchange words per row block, two buffers
+size_t sell_smem_limit(int per);
+bool sell_fits(int per, size_t smem);
+cudaError_t launch_sell(const SoloArgs& a, int per, size_t smem, cudaStream_t s);
 
 cudaError_t prepare_lane_loop(int max_ld);
 int lane_loop_grid(int max_ld);
