@@ -241,11 +241,9 @@ int ubqp_solve_batched(int32_t num, const int64_t* n, const double* const* Q,
  *   row-major, h_out batch (may be NULL), g_out batch x n (may be NULL).
  * 1 <= n <= 65536 and one point must fit in shared memory (n * element size <= 227 KiB,
  * else UBQP_ENOTSUP).  stream: cudaStream_t (NULL = default).
- * Runs the kernel of the inner loop's matrix-vector products (the lock-step GEMV kernel:
- * the same row dot with compensated FP32 sums, here on the caller's rows) with the
- * gradient epilogue; the FP64 dtype runs the same kernel source on FP64 data.  h is summed
- * in FP64.  Scratch (descriptors, work items, partial sums) is allocated and freed on
- * `stream` inside the call; returns after synchronizing `stream`.
+ * FP32 products are summed as in the inner loop's row dots (chains of four, TwoSum-compensated);
+ * h is summed from pairs or in FP64.  Scratch (the row tiles' shares of h) is allocated and freed
+ * on `stream` inside the call; returns after synchronizing `stream`.
  */
 int ubqp_penalized_eval(const void* Q, const void* b, const void* p, const void* x, int64_t n,
                         int64_t batch, int dtype, void* h_out, void* g_out, void* stream);

@@ -286,8 +286,7 @@ def _make_autograd():
 
     class PenalizedObjective(torch.autograd.Function):
         """h(x, p) = x^T Q x + b^T x + sum_i p_i (x_i - x_i^2) (Sec. 4.1, problem (p)).
-        Forward runs ubqp_penalized_eval (the inner loop's GEMV kernel with the gradient
-        epilogue) and keeps g; backward runs ubqp_penalized_vjp: grad_out * g for x,
+        Forward runs ubqp_penalized_eval and keeps g; backward runs ubqp_penalized_vjp: grad_out * g for x,
         sum grad_out * (x - x^2) for p and sum grad_out * x for b.  Q is data (no gradient)."""
 
         @staticmethod

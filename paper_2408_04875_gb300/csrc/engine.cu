@@ -2106,15 +2106,6 @@ int ubqp_initial_point(const double* Q, const double* b, const double* mu, int64
     return rc;
 }
 
-// the rows per work item of a gradient launch: the smallest power of two from 8 that keeps
-// the items of all points within about 8 per SM (at most 256, one epilogue thread per row)
-static int grad_rows_per_item(int64_t n, int64_t batch, int sms)
-{
-    int rb = 8;
-    while (rb < 256 && batch * n / rb > 8 * (int64_t)sms) rb *= 2;
-    return rb;
-}
-
 static int check_grad_args(const char* who, const void* Q, const void* b, const void* p, const void* x, int64_t n,
                            int64_t batch, int dtype, const void* h_out, const void* g_out, bool need_dev)
 {
@@ -2153,40 +2144,26 @@ int ubqp_penalized_eval(const void* Q, const void* b, const void* p, const void*
     int dev = 0, sms = 148;
     UBQP_CK(cudaGetDevice(&dev));
     UBQP_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int rb = grad_rows_per_item(n, batch, sms);
-    const int64_t nblk = (n + rb - 1) / rb;
-    if (batch * nblk > INT32_MAX) {
+    // the calls this entry point refuses, by a count of row blocks: 8 rows, doubled up to 256 while
+    // the blocks of all points exceed 8 per SM
+    int rb = 8;
+    while (rb < 256 && batch * n / rb > 8 * (int64_t)sms) rb *= 2;
+    if (batch * ((n + rb - 1) / rb) > INT32_MAX) {
         set_error("ubqp_penalized_eval: batch x row blocks exceeds 2^31");
         return UBQP_EINVAL;
     }
-    const size_t bytes_lanes = round_up((size_t)batch * sizeof(LaneDev), 256);
-    const size_t bytes_items = round_up((size_t)(batch * nblk) * sizeof(int2), 256);
-    const size_t bytes_queue = 256;
-    const size_t bytes_part = (size_t)(batch * nblk) * sizeof(Partial);
-    char* scratch = nullptr;
-    UBQP_CK(cudaMallocAsync((void**)&scratch, bytes_lanes + bytes_items + bytes_queue + bytes_part, s));
+    const size_t bytes = h_out ? grad_scratch_bytes(n, batch) : 0;
+    void* scratch = nullptr;
     AsyncTemp guard;
-    guard.hold(scratch, s);
-    LaneDev* d_lanes = reinterpret_cast<LaneDev*>(scratch);
-    int2* d_items = reinterpret_cast<int2*>(scratch + bytes_lanes);
-    int32_t* d_queue = reinterpret_cast<int32_t*>(scratch + bytes_lanes + bytes_items);
-    Partial* d_part = reinterpret_cast<Partial*>(scratch + bytes_lanes + bytes_items + bytes_queue);
-    UBQP_CK(launch_grad_setup(d_lanes, d_items, d_queue, d_part, Q, b, p, x, g_out, (int)n, (int)batch, (int)nblk,
-                              (int)es, s));
-    TickArgs ta;
-    memset(&ta, 0, sizeof(ta));
-    ta.lanes = d_lanes;
-    ta.items = d_items;
-    ta.nitems = (int)(batch * nblk);
-    ta.rows_per_item = rb;
-    ta.nlanes = (int)batch;
-    ta.max_ld = (int)n;
-    ta.work = d_queue;
-    ta.done = d_queue + 1;
-    UBQP_CK(launch_phase_a_grad(ta, dtype, n, s));
-    if (h_out) UBQP_CK(launch_grad_reduce(d_lanes, (int)batch, h_out, dtype, s));
-    guard.release();
-    UBQP_CK(cudaFreeAsync(scratch, s));
+    if (bytes > 0) {
+        UBQP_CK(cudaMallocAsync(&scratch, bytes, s));
+        guard.hold(scratch, s);
+    }
+    UBQP_CK(launch_grad(Q, b, p, x, n, batch, dtype, h_out, g_out, scratch, sms, s));
+    if (scratch) {
+        guard.release();
+        UBQP_CK(cudaFreeAsync(scratch, s));
+    }
     UBQP_CK(cudaStreamSynchronize(s));
     return UBQP_OK;
 }

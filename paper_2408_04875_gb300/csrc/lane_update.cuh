@@ -679,7 +679,6 @@ static __device__ __noinline__ void lane_update(const LaneDev& L, const Params& 
     // descriptor fields read once, before any store (the compiler cannot rule out that the
     // stores through vec alias the descriptor and would load them again after each)
     const int mode = L.mode, ld = L.ld;
-    if (mode == MODE_GRAD) return;
     float* const vec = L.vec;
     __nv_bfloat16* const u_hi = L.u_hi;
     __nv_bfloat16* const u_lo = L.u_lo;

@@ -5,12 +5,10 @@
 // computation as ubqp_penalized_eval, with the same kernel and the same work partition,
 // with its scratch in a fixed static device array.
 //
-// The scratch (per-point descriptors, work items, the work-queue counters, per-block
-// partial sums) lives in g_noalloc_scratch below.  Every GPU that loads the library holds
-// it until the process exits.  All calls share it and it keeps the last call's contents;
-// each call rewrites every byte it later reads (the queue counters are cleared by the
-// call's set-up kernel), so nothing has to start at zero.  Calls that overlap on the GPU
-// (other streams, other host threads) race on it.
+// The scratch (the row tiles' shares of h) lives in g_noalloc_scratch below.  Every GPU that loads
+// the library holds it until the process exits.  All calls share it and it keeps the last call's
+// contents; each call writes every word it later reads, so nothing has to start at zero.  Calls
+// that overlap on the GPU (other streams, other host threads) race on it.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -24,17 +22,9 @@ namespace ubqp {
 
 constexpr int kNoallocMaxLanes = 256;
 constexpr int kNoallocMaxItems = 16384;
-constexpr size_t kLanesBytes = (size_t)kNoallocMaxLanes * 320;   // room for one descriptor per point
-static_assert(sizeof(LaneDev) <= 320, "descriptor outgrew its scratch slot");
-constexpr size_t kItemsBytes = (size_t)kNoallocMaxItems * sizeof(int2);
-constexpr size_t kQueueBytes = 256;
-constexpr size_t kPartBytes = (size_t)kNoallocMaxItems * sizeof(Partial);
-constexpr size_t kLanesOff = 0;
-constexpr size_t kItemsOff = (kLanesBytes + 255) / 256 * 256;
-constexpr size_t kQueueOff = kItemsOff + (kItemsBytes + 255) / 256 * 256;
-constexpr size_t kPartOff = kQueueOff + kQueueBytes;
-constexpr size_t kScratchBytes = kPartOff + kPartBytes;
-static_assert(kScratchBytes == UBQP_NOALLOC_SCRATCH_BYTES, "header and scratch layout disagree");
+constexpr size_t kScratchBytes = UBQP_NOALLOC_SCRATCH_BYTES;
+// the limits below admit at most kNoallocMaxItems blocks of 256 rows, i.e. this many tiles of 32
+static_assert(((size_t)kNoallocMaxItems * 8 + kNoallocMaxLanes) * sizeof(double) <= kScratchBytes, "shares of h fit");
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
@@ -138,7 +128,7 @@ extern "C" int ubqp_penalized_eval_noalloc(const void* Q, const void* b, const v
         set_error("ubqp_penalized_eval_noalloc: %s", cudaGetErrorString(cudaGetLastError()));
         return UBQP_ECUDA;
     }
-    // the work partition of ubqp_penalized_eval (same rows per item), so both return the same values
+    // (the kernel and its partition are those of ubqp_penalized_eval, so both return the same values)
     int rb = 8;
     while (rb < 256 && batch * n / rb > 8 * (int64_t)sms) rb *= 2;
     const int64_t nblk = (n + rb - 1) / rb;
@@ -164,24 +154,8 @@ extern "C" int ubqp_penalized_eval_noalloc(const void* Q, const void* b, const v
         set_error("ubqp_penalized_eval_noalloc: resolving the scratch array failed: %s", cudaGetErrorString(e));
         return UBQP_ECUDA;
     }
-    unsigned char* base = static_cast<unsigned char*>(scratch);
     cudaStream_t s = (cudaStream_t)stream;
-    const int nitems = (int)(batch * nblk);
-    e = launch_grad_setup(reinterpret_cast<LaneDev*>(base + kLanesOff), reinterpret_cast<int2*>(base + kItemsOff),
-                          reinterpret_cast<int32_t*>(base + kQueueOff), reinterpret_cast<Partial*>(base + kPartOff), Q, b,
-                          p, x, g_out, (int)n, (int)batch, (int)nblk, (int)es, s);
-    TickArgs ta;
-    memset(&ta, 0, sizeof(ta));
-    ta.lanes = reinterpret_cast<const LaneDev*>(base + kLanesOff);
-    ta.items = reinterpret_cast<const int2*>(base + kItemsOff);
-    ta.nitems = nitems;
-    ta.rows_per_item = rb;
-    ta.nlanes = (int)batch;
-    ta.max_ld = (int)n;
-    ta.work = reinterpret_cast<int32_t*>(base + kQueueOff);
-    ta.done = ta.work + 1;
-    if (e == cudaSuccess) e = launch_phase_a_grad(ta, dtype, n, s);
-    if (e == cudaSuccess && h_out) e = launch_grad_reduce(ta.lanes, (int)batch, h_out, dtype, s);
+    e = launch_grad(Q, b, p, x, n, batch, dtype, h_out, g_out, scratch, sms, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
         set_error("ubqp_penalized_eval_noalloc: %s", cudaGetErrorString(e));

@@ -29,10 +29,9 @@ enum Phase : int32_t {
     PH_LOB_INIT = 3,  // first matvec of the lambda_min solver (A x_0)
     PH_LOB = 4,       // one LOBPCG iteration for lambda_min of Z^-1/2 Qbar_II Z^-1/2
     PH_INNER = 5,     // one iteration of Alg. 2 (PABB) or Alg. 1 (PPA)
-    PH_GRAD = 6,      // stand-alone h and gradient (penalized_eval)
 };
 
-enum LaneMode : int32_t { MODE_GEMV = 0, MODE_TC = 1, MODE_GRAD = 2 };
+enum LaneMode : int32_t { MODE_GEMV = 0, MODE_TC = 1 };
 
 // stop hooks used by the test entry points
 enum StopAfter : int32_t { STOP_INNER = 1, STOP_LOB = 2, STOP_JACOBI = 4 };
@@ -61,7 +60,7 @@ enum Vec : int32_t {
 struct __align__(16) Partial {
     float2 s[12];   // compensated sums (hi, lo)
     float m[6];     // maxima (all values >= 0)
-    double f;       // FP64 sum (objective of a rounded point / h of penalized_eval)
+    double f;       // FP64 sum (objective of a rounded point)
 };
 static_assert(sizeof(Partial) == 128, "Partial must stay 128 bytes");
 
@@ -120,13 +119,7 @@ struct LaneDev {
     float* trace_alpha;
     float qmax_off;        // max_{i != j} |Q'_ij|
     float rabs_max;        // max_i rabs_i
-    // gradient lanes (penalized_eval)
-    const void* gQ;
-    const void* gb;
-    const void* gp;
-    const void* gx;
-    void* gg;
-    int32_t gld;
+    int32_t pad_;
     int32_t spwps;         // sliced storage: warps per 32-row slice (8 / slices per item)
     int32_t* nt_active;    // TC lanes: unfinished lanes of this lane's N tile (decremented
                            // by the update that finishes the lane), else null
@@ -445,7 +438,6 @@ struct TickArgs {
 cudaError_t prepare_phase_a_gemv(int max_ld);
 int gemv_grid(int max_ld, int nitems);
 cudaError_t launch_phase_a_gemv_f32(const TickArgs& a, cudaStream_t s);
-cudaError_t launch_phase_a_grad(const TickArgs& a, int dtype, int64_t n, cudaStream_t s);
 constexpr int kSymT = 128;   // tile edge of the symmetric storage
 constexpr int kSymGroup = 2; // tiles per first-stage ring entry
 
@@ -530,10 +522,10 @@ cudaError_t prepare_lane_loop(int max_ld);
 int lane_loop_grid(int max_ld);
 cudaError_t launch_lane_loop(const LoopArgs& a, cudaStream_t s);   // seed + loop kernels
 cudaError_t launch_phase_b(const TickArgs& a, int32_t* active_count, cudaStream_t s);
-cudaError_t launch_grad_reduce(const LaneDev* lanes, int nlanes, void* h_out, int dtype,
-                               cudaStream_t s);
-cudaError_t launch_grad_setup(LaneDev* lanes, int2* items, int32_t* queue, Partial* part, const void* Q, const void* b,
-                              const void* p, const void* x, void* g, int n, int batch, int nblk, int es, cudaStream_t s);
+// penalized objective and gradient (grad.cu): scratch of grad_scratch_bytes(n, batch) when h is wanted
+size_t grad_scratch_bytes(int64_t n, int64_t batch);
+cudaError_t launch_grad(const void* Q, const void* b, const void* p, const void* x, int64_t n, int64_t batch, int dtype,
+                        void* h, void* g, void* scratch, int sms, cudaStream_t s);
 cudaError_t launch_penalized_vjp(const void* x, const void* g, const void* go, int64_t n, int64_t batch, int dtype,
                                  void* gx, void* gp, void* gb, cudaStream_t s);
 
