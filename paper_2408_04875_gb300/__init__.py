@@ -72,6 +72,8 @@ class Opts(C.Structure):
 def lib():
     """The loaded CUDA library; raises if it has not been built."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(LIB_PATH):
@@ -140,6 +142,17 @@ def _as_f64(a, keep):
     arr = np.ascontiguousarray(a, dtype=np.float64)
     keep.append(arr)
     return arr.ctypes.data
+
+
+def _dense(t, dt):
+    """A tensor's data as contiguous dt (itself when it is that already)."""
+    if t is None or (t.dtype == dt and t.is_contiguous()):
+        return t
+    return t.to(dt).contiguous()
+
+
+def _dptr(t):
+    return None if t is None else t.data_ptr()
 
 
 def _ptr_array(ptrs, keep):
@@ -239,16 +252,12 @@ def penalized_eval(Q, b, p, x, want_h: bool = True, want_g: bool = True, stream=
     squeeze = x.dim() == 1
     X = x.reshape(1, -1) if squeeze else x
     n = Q.shape[0]
-    Qc = Q.contiguous()
-    Xc = X.to(dt).contiguous()
-    bc = None if b is None else b.to(dt).contiguous()
-    pc = None if p is None else p.to(dt).contiguous()
+    Qc, Xc, bc, pc = _dense(Q, dt), _dense(X, dt), _dense(b, dt), _dense(p, dt)
     h = torch.empty(Xc.shape[0], dtype=dt, device=Q.device) if want_h else None
     g = torch.empty_like(Xc) if want_g else None
     s = stream if stream is not None else torch.cuda.current_stream(Q.device).cuda_stream
-    rc = lib().ubqp_penalized_eval(Qc.data_ptr(), None if bc is None else bc.data_ptr(),
-                                   None if pc is None else pc.data_ptr(), Xc.data_ptr(), n, Xc.shape[0], code,
-                                   None if h is None else h.data_ptr(), None if g is None else g.data_ptr(), s)
+    rc = lib().ubqp_penalized_eval(Qc.data_ptr(), _dptr(bc), _dptr(pc), Xc.data_ptr(), n, Xc.shape[0], code, _dptr(h),
+                                   _dptr(g), s)
     _check(rc, "ubqp_penalized_eval")
     if squeeze:
         h = None if h is None else h[0]
@@ -265,16 +274,15 @@ def penalized_vjp(x, g, grad_h, want_x=True, want_p=False, want_b=False, stream=
     X = x.reshape(1, -1) if squeeze else x
     dt = X.dtype
     code = 1 if dt == torch.float64 else 0
-    Xc = X.contiguous()
-    Gc = g.reshape(Xc.shape).to(dt).contiguous()
-    go = grad_h.reshape(-1).to(dt).contiguous()
+    Xc = _dense(X, dt)
+    Gc = _dense(g if g.shape == Xc.shape else g.reshape(Xc.shape), dt)
+    go = _dense(grad_h if grad_h.dim() == 1 else grad_h.reshape(-1), dt)
     gx = torch.empty_like(Xc) if want_x else None
     gp = torch.empty(Xc.shape[1], dtype=dt, device=Xc.device) if want_p else None
     gb = torch.empty(Xc.shape[1], dtype=dt, device=Xc.device) if want_b else None
     s = stream if stream is not None else torch.cuda.current_stream(Xc.device).cuda_stream
-    rc = lib().ubqp_penalized_vjp(Xc.data_ptr(), Gc.data_ptr(), go.data_ptr(), Xc.shape[1], Xc.shape[0], code,
-                                  None if gx is None else gx.data_ptr(), None if gp is None else gp.data_ptr(),
-                                  None if gb is None else gb.data_ptr(), s)
+    rc = lib().ubqp_penalized_vjp(Xc.data_ptr(), Gc.data_ptr(), go.data_ptr(), Xc.shape[1], Xc.shape[0], code, _dptr(gx),
+                                  _dptr(gp), _dptr(gb), s)
     _check(rc, "ubqp_penalized_vjp")
     if squeeze and gx is not None:
         gx = gx[0]

@@ -84,7 +84,7 @@ struct AsyncTemp {
     void release() { p = nullptr; }
 };
 
-// one device allocation carved into 256-byte aligned pieces
+// one stream-ordered device allocation carved into 256-byte aligned pieces
 class Arena {
   public:
     size_t reserve(size_t bytes)
@@ -93,13 +93,14 @@ class Arena {
         size_ += round_up(bytes ? bytes : 1, 256);
         return off;
     }
-    int commit()
+    int commit(cudaStream_t s)
     {
         if (size_ == 0) return UBQP_OK;
-        cudaError_t e = cudaMalloc(&base_, size_);
+        stream_ = s;
+        cudaError_t e = work_alloc(&base_, size_, s);
         if (e != cudaSuccess) {
             cudaGetLastError();
-            set_error("cudaMalloc of %zu bytes failed: %s", size_, cudaGetErrorString(e));
+            set_error("allocation of %zu bytes failed: %s", size_, cudaGetErrorString(e));
             base_ = nullptr;
             return e == cudaErrorMemoryAllocation ? UBQP_ENOMEM : UBQP_ECUDA;
         }
@@ -111,13 +112,15 @@ class Arena {
         return reinterpret_cast<T*>(static_cast<char*>(base_) + off);
     }
     size_t size() const { return size_; }
-    ~Arena()
+    void release()   // while the stream lives
     {
-        if (base_) cudaFree(base_);
+        if (base_) cudaFreeAsync(base_, stream_);
+        base_ = nullptr;
     }
 
   private:
     void* base_ = nullptr;
+    cudaStream_t stream_ = nullptr;
     size_t size_ = 0;
 };
 
@@ -266,12 +269,17 @@ class Solver {
     {
         if (gexec_) cudaGraphExecDestroy(gexec_);
         if (graph_) cudaGraphDestroy(graph_);
-        if (h_active_) cudaFreeHost(h_active_);
+        if (h_active_) {
+            cudaStreamSynchronize(stream_);   // a copy into it may be in flight
+            pinned_put(h_active_);
+        }
         if (ev0_) cudaEventDestroy(ev0_);
         if (ev1_) cudaEventDestroy(ev1_);
         for (auto e : evA_) cudaEventDestroy(e);
         if (stream_) {
             cudaStreamSynchronize(stream_);
+            ar_.release();
+            sp_ar_.release();
             cudaStreamDestroy(stream_);
         }
     }
@@ -318,7 +326,7 @@ class Solver {
                 cnt[t] = c;
             }
             if (any_dev) {
-                UBQP_CK(cudaMallocAsync((void**)&dcnt, insts.size() * sizeof(unsigned long long), stream_));
+                UBQP_CK(work_alloc((void**)&dcnt, insts.size() * sizeof(unsigned long long), stream_));
                 guard.hold(dcnt, stream_);
                 UBQP_CK(cudaMemsetAsync(dcnt, 0, insts.size() * sizeof(unsigned long long), stream_));
                 for (size_t t = 0; t < insts.size(); ++t)
@@ -393,9 +401,11 @@ class Solver {
         o_valid_ = ar_.reserve(insts.size() * 4 * sizeof(float));
         o_nnz_ = ar_.reserve(insts.size() * sizeof(unsigned long long));
         o_inexact_ = ar_.reserve(insts.size() * sizeof(int));
-        o_hist_ = ar_.reserve(UBQP_HIST_BINS * sizeof(int64_t));
+        // histogram, bytes and flops side by side: one clear, one copy back
+        o_hist_ = ar_.reserve((UBQP_HIST_BINS + 2) * sizeof(int64_t));
+        o_bytes_ = o_hist_ + UBQP_HIST_BINS * sizeof(int64_t);
+        o_flops_ = o_bytes_ + sizeof(unsigned long long);
         o_active_ = ar_.reserve(sizeof(int32_t));
-        o_bytes_ = ar_.reserve(sizeof(unsigned long long));
 
         lane_inst_.resize(lanes.size());
         for (size_t l = 0; l < lanes.size(); ++l) lane_inst_[l] = lanes[l].inst;
@@ -525,7 +535,6 @@ class Solver {
             o_tcinst_ = ar_.reserve(inst_.size() * sizeof(TcInst));
             o_tcerr_ = ar_.reserve(sizeof(int32_t));
         }
-        o_flops_ = ar_.reserve(sizeof(unsigned long long));
         o_states_ = ar_.reserve(lanes.size() * sizeof(LaneState));
         o_counters_ = ar_.reserve(lanes.size() * sizeof(unsigned int));
         o_symctr_ = sym_ ? ar_.reserve(lanes.size() * sizeof(unsigned int)) : 0;
@@ -580,11 +589,9 @@ class Solver {
                 o_budget_ = ar_.reserve(lanes.size() * sizeof(int32_t));
             }
         }
-        rc = ar_.commit();
+        rc = ar_.commit(stream_);
         if (rc) return rc;
-        UBQP_CK(cudaMemsetAsync(ar_.at<char>(o_hist_), 0, UBQP_HIST_BINS * sizeof(int64_t), stream_));
-        UBQP_CK(cudaMemsetAsync(ar_.at<char>(o_bytes_), 0, sizeof(unsigned long long), stream_));
-        UBQP_CK(cudaMemsetAsync(ar_.at<char>(o_flops_), 0, sizeof(unsigned long long), stream_));
+        UBQP_CK(cudaMemsetAsync(ar_.at<char>(o_hist_), 0, (UBQP_HIST_BINS + 2) * sizeof(int64_t), stream_));
         UBQP_CK(cudaMemsetAsync(ar_.at<char>(o_counters_), 0, lanes.size() * sizeof(unsigned int), stream_));
         if (sym_) UBQP_CK(cudaMemsetAsync(ar_.at<char>(o_symctr_), 0, lanes.size() * sizeof(unsigned int), stream_));
         UBQP_CK(cudaMemsetAsync(ar_.at<char>(o_queue_), 0, 2 * sizeof(int32_t), stream_));
@@ -914,7 +921,7 @@ class Solver {
             cluster_tuned_ = 2;
         } else {
             float* raw = nullptr;
-            UBQP_CK(cudaMallocAsync((void**)&raw, raw_elems * sizeof(float), stream_));
+            UBQP_CK(work_alloc((void**)&raw, raw_elems * sizeof(float), stream_));
             AsyncTemp guard;
             guard.hold(raw, stream_);
             TcArgs a;
@@ -1019,7 +1026,7 @@ class Solver {
         const bool prof = o_.profile_kernels != 0;
         if (prof) ta.P.bytes = ar_.at<unsigned long long>(o_bytes_);
         int32_t* d_active = ar_.at<int32_t>(o_active_);
-        UBQP_CK(cudaMallocHost(&h_active_, sizeof(int32_t)));
+        UBQP_CK(pinned_get((void**)&h_active_));
         if (!tc_ && nitems_ > 0) {
             UBQP_CK(prepare_phase_a_gemv(max_ld_));
             ta.grid = gemv_grid(max_ld_, nitems_);
@@ -1061,7 +1068,7 @@ class Solver {
             if (timeline) {
                 g_tl_ms.clear();
                 g_tl_work.clear();
-                UBQP_CK(cudaMallocAsync((void**)&d_snap, (size_t)T * sizeof(unsigned long long), stream_));
+                UBQP_CK(work_alloc((void**)&d_snap, (size_t)T * sizeof(unsigned long long), stream_));
                 snap_guard.hold(d_snap, stream_);
             }
         }
@@ -1210,7 +1217,7 @@ class Solver {
             nsl_total += (size_t)(inst_[t].n + 31) / 32;
         }
         int32_t* dw = nullptr;
-        UBQP_CK(cudaMallocAsync((void**)&dw, std::max<size_t>(nsl_total, 1) * sizeof(int32_t), stream_));
+        UBQP_CK(work_alloc((void**)&dw, std::max<size_t>(nsl_total, 1) * sizeof(int32_t), stream_));
         AsyncTemp guard;
         guard.hold(dw, stream_);
         for (size_t t = 0; t < inst_.size(); ++t)
@@ -1235,7 +1242,7 @@ class Solver {
             I.max_width = ns ? *std::max_element(w.begin() + sl0[t], w.begin() + sl0[t] + ns) : 0;
             sliced_entries_ += (int64_t)entries;
         }
-        int rc = sp_ar_.commit();
+        int rc = sp_ar_.commit(stream_);
         if (rc) return rc;
         for (size_t t = 0; t < inst_.size(); ++t) {
             InstDev& I = inst_[t];
@@ -1287,7 +1294,7 @@ class Solver {
         const bool prof = o_.profile_kernels != 0;
         if (prof) sa.P.bytes = ar_.at<unsigned long long>(o_bytes_);
         UBQP_CK(prepare_solo(max_ld_, solo_one_ok_));
-        UBQP_CK(cudaMallocHost(&h_active_, 2 * sizeof(int32_t)));
+        UBQP_CK(pinned_get((void**)&h_active_));
         if (prof) {
             evA_.resize(2);
             for (auto& e : evA_) UBQP_CK(cudaEventCreate(&e));
@@ -1508,7 +1515,7 @@ class Solver {
         la.P = make_params(o_, ar_.at<int64_t>(o_hist_));
         const bool prof = o_.profile_kernels != 0;
         if (prof) la.P.bytes = ar_.at<unsigned long long>(o_bytes_);
-        UBQP_CK(cudaMallocHost(&h_active_, sizeof(int32_t)));
+        UBQP_CK(pinned_get((void**)&h_active_));
         if (prof) {
             evA_.resize(2);
             for (auto& e : evA_) UBQP_CK(cudaEventCreate(&e));
@@ -1626,9 +1633,12 @@ class Solver {
     int fill_stats(ubqp_stats* s)
     {
         if (!s) return UBQP_OK;
-        std::vector<LaneState> st;
-        int rc = states(st);
-        if (rc) return rc;
+        std::vector<LaneState> st(nlanes_);
+        int64_t ctr[UBQP_HIST_BINS + 2];
+        UBQP_CK(cudaMemcpyAsync(ctr, ar_.at<int64_t>(o_hist_), sizeof(ctr), cudaMemcpyDeviceToHost, stream_));
+        UBQP_CK(cudaMemcpyAsync(st.data(), ar_.at<LaneState>(o_states_), nlanes_ * sizeof(LaneState),
+                                cudaMemcpyDeviceToHost, stream_));
+        UBQP_CK(cudaStreamSynchronize(stream_));
         memset(s, 0, sizeof(*s));
         for (int l = 0; l < nlanes_; ++l) {
             const LaneState& S = st[l];
@@ -1653,16 +1663,10 @@ class Solver {
         s->ms_device = ms_device_;
         s->phase_a_ms = phase_a_ms_;
         s->phase_a_launches = phase_a_launches_;
-        unsigned long long by = 0;
-        UBQP_CK(cudaMemcpyAsync(&by, ar_.at<unsigned long long>(o_bytes_), sizeof(by), cudaMemcpyDeviceToHost, stream_));
-        UBQP_CK(cudaStreamSynchronize(stream_));
-        s->phase_a_bytes = (int64_t)by;
+        s->phase_a_bytes = ctr[UBQP_HIST_BINS];
         s->kernel_launches = launches_;
         s->ms_to_target = ms_to_target_;
-        unsigned long long fl = 0;
-        UBQP_CK(cudaMemcpyAsync(&fl, ar_.at<unsigned long long>(o_flops_), sizeof(fl), cudaMemcpyDeviceToHost, stream_));
-        UBQP_CK(cudaStreamSynchronize(stream_));
-        s->phase_a_flops = (int64_t)fl;
+        s->phase_a_flops = ctr[UBQP_HIST_BINS + 1];
         s->cluster_size = tc_ ? tc_S_ : 0;
         s->cluster_tuned = cluster_tuned_;
         for (int c = 0; c < 9; ++c) s->cluster_probe_us[c] = cluster_probe_us_[c];
@@ -1670,9 +1674,7 @@ class Solver {
         s->sym_storage = sym_ ? 1 : 0;
         s->storage = tc_ ? 3 : (sparse_ ? 2 : (sym_ ? 1 : 0));
         s->gemv_kernel = tc_ ? 0 : (solo_ ? 3 : (loop_ ? 2 : 1));
-        UBQP_CK(cudaMemcpyAsync(s->inner_hist, ar_.at<int64_t>(o_hist_), sizeof(s->inner_hist), cudaMemcpyDeviceToHost,
-                                stream_));
-        UBQP_CK(cudaStreamSynchronize(stream_));
+        memcpy(s->inner_hist, ctr, sizeof(s->inner_hist));
         return UBQP_OK;
     }
 
@@ -1684,7 +1686,7 @@ class Solver {
         double* tmp = nullptr;
         AsyncTemp guard;
         if (host) {
-            UBQP_CK(cudaMallocAsync((void**)&tmp, (size_t)n * 8, stream_));
+            UBQP_CK(work_alloc((void**)&tmp, (size_t)n * 8, stream_));
             guard.hold(tmp, stream_);
             dst = tmp;
         }
@@ -1708,7 +1710,7 @@ class Solver {
             double* tmp = nullptr;
             AsyncTemp guard;
             if (host) {
-                UBQP_CK(cudaMallocAsync((void**)&tmp, (size_t)cnt * 8, stream_));
+                UBQP_CK(work_alloc((void**)&tmp, (size_t)cnt * 8, stream_));
                 guard.hold(tmp, stream_);
                 d = tmp;
             }
@@ -2156,7 +2158,7 @@ int ubqp_penalized_eval(const void* Q, const void* b, const void* p, const void*
     void* scratch = nullptr;
     AsyncTemp guard;
     if (bytes > 0) {
-        UBQP_CK(cudaMallocAsync(&scratch, bytes, s));
+        UBQP_CK(work_alloc(&scratch, bytes, s));
         guard.hold(scratch, s);
     }
     UBQP_CK(launch_grad(Q, b, p, x, n, batch, dtype, h_out, g_out, scratch, sms, s));

@@ -29,12 +29,9 @@ static_assert(((size_t)kNoallocMaxItems * 8 + kNoallocMaxLanes) * sizeof(double)
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
 // Device address of g_noalloc_scratch in each CUDA context that has used this entry point.
-// The key is the context's unique ID (cuCtxGetId), not the device index: after a device
+// The key is the context's unique ID (current_context_id), not the device index: after a device
 // reset the runtime creates a new primary context, reloads the module, and the array may
 // live at another address; the new context has a new ID, so its address is resolved again.
-typedef CUresult (*PFN_ctx_current)(CUcontext*);
-typedef CUresult (*PFN_ctx_id)(CUcontext, unsigned long long*);
-
 static std::mutex g_noalloc_mu;
 struct ScratchAddr {
     unsigned long long ctx_id;
@@ -43,36 +40,11 @@ struct ScratchAddr {
 static ScratchAddr g_noalloc_addr[64];
 static int g_noalloc_next = 0;
 
-template <class F>
-static F driver_fn(const char* name)
-{
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion(name, &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess) {
-        cudaGetLastError();
-        return nullptr;
-    }
-    return reinterpret_cast<F>(p);
-}
-
 static cudaError_t noalloc_scratch(void** out)
 {
-    static PFN_ctx_current ctx_current = driver_fn<PFN_ctx_current>("cuCtxGetCurrent");
-    static PFN_ctx_id ctx_id = driver_fn<PFN_ctx_id>("cuCtxGetId");
-    if (!ctx_current || !ctx_id) return cudaErrorNotSupported;
-    CUcontext ctx = nullptr;
     unsigned long long id = 0;
-    if (ctx_current(&ctx) == CUDA_SUCCESS && !ctx) {
-        // no context current on this thread yet: make the device's primary context current
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaSetDevice(dev);
-        if (e != cudaSuccess) return e;
-        if (ctx_current(&ctx) != CUDA_SUCCESS) ctx = nullptr;
-    }
-    if (!ctx || ctx_id(ctx, &id) != CUDA_SUCCESS) return cudaErrorDeviceUninitialized;
-    cudaError_t e;
+    cudaError_t e = current_context_id(&id);
+    if (e != cudaSuccess) return e;
     std::lock_guard<std::mutex> lk(g_noalloc_mu);
     for (const ScratchAddr& a : g_noalloc_addr)
         if (a.addr && a.ctx_id == id) {

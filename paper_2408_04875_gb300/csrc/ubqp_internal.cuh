@@ -529,6 +529,13 @@ cudaError_t launch_grad(const void* Q, const void* b, const void* p, const void*
 cudaError_t launch_penalized_vjp(const void* x, const void* g, const void* go, int64_t n, int64_t batch, int dtype,
                                  void* gx, void* gp, void* gb, cudaStream_t s);
 
+// device scratch and pinned words kept between calls (workspace.cu); free the former with
+// cudaFreeAsync on a stream ordered after its last use
+cudaError_t current_context_id(unsigned long long* id);
+cudaError_t work_alloc(void** p, size_t bytes, cudaStream_t s);
+cudaError_t pinned_get(void** p);   // 64 bytes
+void pinned_put(void* p);
+
 // the calling thread's last-error text (ubqp_last_error), shared by every entry point
 void set_error(const char* fmt, ...);
 void clear_error();
