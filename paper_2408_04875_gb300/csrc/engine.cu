@@ -437,6 +437,16 @@ class Solver {
             return UBQP_ENOTSUP;
         }
         solo_ = solo_fit && (o_.gemv_kernel == 3 || (solo_auto && (lanes.size() == 1 || sparse_)));
+        // lanes on the symmetric tiles (dense data): groups too, while a CTA owns few tiles
+        symg_ = false;
+        if (sym_ && o_.gemv_kernel == 0) {
+            std::vector<int> ids(lanes.size());
+            for (size_t l = 0; l < lanes.size(); ++l) ids[l] = (int)l;
+            int32_t mat = 0;
+            symg_ = plan_sym_groups(ids) && sym_lane_smem(max_ld, kSymMaxTiles, &mat) > 0;
+            solo_ = symg_;
+            solo_capc_ = symg_ ? num_sms_ : 0;
+        }
         if (solo_ && lanes.size() == 1 && sparse_) {
             // one CTA per 32-row slice (one CTA for up to 256 rows), unless the caller chose
             const int n0 = (int)insts[lanes[0].inst].n;
@@ -451,7 +461,9 @@ class Solver {
         } else if (solo_ && lanes.size() == 1) {
             solo_shape((int)insts[lanes[0].inst].n, o_.rows_per_item, num_sms_, &solo_grid_, &rb, &solo_nblk_);
         }
-        if (solo_ && lanes.size() > 1) {
+        if (symg_) {
+            // planned above
+        } else if (solo_ && lanes.size() > 1) {
             solo_nb_.assign(lanes.size(), 0);
             std::vector<int> ids(lanes.size());
             for (size_t l = 0; l < lanes.size(); ++l) {
@@ -512,7 +524,8 @@ class Solver {
             // the single-lane kernel's one-barrier steps alternate between two sets of records
             o_part_[l] = ar_.reserve((size_t)(solo_ ? 2 : 1) * L.nblk * sizeof(Partial));
             xch[l] = xch_words;
-            if (solo_ && sparse_) xch_words += (size_t)kSellWordsPerBlock * L.nblk;
+            if (symg_) xch_words += sym_lane_words(I.nb);
+            else if (solo_ && sparse_) xch_words += (size_t)kSellWordsPerBlock * L.nblk;
             if (in.trace_len > 0) {
                 o_trace_x_[l] = ar_.reserve((size_t)in.trace_len * I.n * 4);
                 o_trace_a_[l] = ar_.reserve((size_t)in.trace_len * 4);
@@ -762,8 +775,8 @@ class Solver {
                 L.spc = sp_ar_.at<uint16_t>(I.o_spc);
                 L.spo = sp_ar_.at<int64_t>(I.o_spo);
                 L.spwps = 256 / rows_per_item_;   // 256 threads per GEMV CTA
-                L.xch = solo_ ? ar_.at<ulonglong2>(o_xch) + xch[l] : nullptr;
             }
+            if (solo_ && (sparse_ || symg_)) L.xch = ar_.at<ulonglong2>(o_xch) + xch[l];
             L.Qeval = tc ? nullptr : ar_.at<float2>(I.o_Qeval);
             L.d = ar_.at<float>(I.o_d);
             L.bprime = ar_.at<float>(I.o_bp);
@@ -1272,7 +1285,9 @@ class Solver {
             sa.gcta = sa.gfirst + solo_gmax_ + 1;
             sa.grid = solo_gcta_.back();
             sell_ = sell_shape(&sell_smem_, &sa.mat_bytes);
+            if (symg_) sell_smem_ = sym_lane_smem(max_ld_, sym_group_tiles(), &sa.mat_bytes);
         };
+        sa.sym = symg_ ? ar_.at<SymLane>(o_symlanes_) : nullptr;
         if (nlanes_ > 1 && sparse_) {   // the widths are known now: the plan whose slices fit best
             std::vector<int> ids(nlanes_);
             for (int l = 0; l < nlanes_; ++l) ids[l] = l;
@@ -1307,7 +1322,8 @@ class Solver {
         for (;;) {
             UBQP_CK(cudaMemsetAsync(sa.active_after, 0, sizeof(int32_t), stream_));
             if (prof) UBQP_CK(cudaEventRecord(evA_[0], stream_));
-            if (sell_) UBQP_CK(launch_sell(sa, solo_per_, sell_smem_, stream_));
+            if (symg_) UBQP_CK(launch_sym(sa, sell_smem_, stream_));
+            else if (sell_) UBQP_CK(launch_sell(sa, solo_per_, sell_smem_, stream_));
             else UBQP_CK(launch_solo(sa, max_ld_, stream_));
             if (prof) UBQP_CK(cudaEventRecord(evA_[1], stream_));
             UBQP_CK(cudaMemcpyAsync(h_active_, ctl, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, stream_));
@@ -1344,7 +1360,7 @@ class Solver {
                 std::vector<int> ids;
                 for (int l = 0; l < nlanes_; ++l)
                     if (st[l].phase != PH_DONE) ids.push_back(l);
-                if (!ids.empty() && plan_solo_groups(ids, max_ld_, true)) {
+                if (!ids.empty() && (symg_ ? plan_sym_groups(ids) : plan_solo_groups(ids, max_ld_, true))) {
                     UBQP_CK(upload_solo_plan());
                     set_plan();
                 }
@@ -1434,6 +1450,44 @@ class Solver {
         solo_gcta_ = gc;
         solo_max_lanes_ = std::max(solo_max_lanes_, max_lanes);
         return true;
+    }
+
+    // Groups of CTAs (one per SM) for lanes on the symmetric tiles, largest first: ceil(tiles / m) CTAs
+    // each, at least one per row block, for the smallest m (tiles per CTA) at which all groups are
+    // resident together.  Device time against the lane loop (three subproblems of at most 40 steps):
+    // 4 lanes of n = 2000 (m = 4) 2.3 against 6.4 ms, 8 of them (m = 8) 3.5 against 6.9 ms, 4 of
+    // n = 4500 (m = 18) 7.5 against 10.4 ms; beyond kSymMaxTiles the lane loop keeps all SMs busier
+    bool plan_sym_groups(const std::vector<int>& ids)
+    {
+        auto tiles = [&](int l) { const int nb = inst_[(size_t)lane_inst_[l]].nb; return nb * (nb + 1) / 2; };
+        auto ctas = [&](int l, int m) { return std::max(inst_[(size_t)lane_inst_[l]].nb, (tiles(l) + m - 1) / m); };
+        std::vector<int> order(ids);
+        std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return tiles(a) > tiles(b); });
+        for (int m = 1; m <= kSymMaxTiles; ++m) {
+            int64_t tot = 0;
+            for (int l : ids) tot += ctas(l, m);
+            if (tot > num_sms_) continue;
+            solo_glanes_.clear();
+            solo_gfirst_.assign(1, 0);
+            solo_gcta_.assign(1, 0);
+            for (int l : order) {
+                solo_glanes_.push_back(l);
+                solo_gfirst_.push_back((int)solo_glanes_.size());
+                solo_gcta_.push_back(solo_gcta_.back() + ctas(l, m));
+            }
+            return true;
+        }
+        return false;
+    }
+    // the most tiles a CTA of the current plan owns
+    int sym_group_tiles() const
+    {
+        int m = 1;
+        for (size_t g = 0; g + 1 < solo_gcta_.size(); ++g) {
+            const int nb = inst_[(size_t)lane_inst_[solo_glanes_[g]]].nb, nc = solo_gcta_[g + 1] - solo_gcta_[g];
+            m = std::max(m, (nb * (nb + 1) / 2 + nc - 1) / nc);
+        }
+        return m;
     }
 
     // Relative cost of a step with `per` CTAs of m slices on an SM: a slice whose entries stay in
@@ -1767,6 +1821,7 @@ class Solver {
     int64_t solo_capc_ = 0;      // CTAs resident at once
     int solo_per_ = 1;           // CTAs of the current plan that share an SM
     bool sell_ = false;          // the current plan runs on the sliced kernel
+    bool symg_ = false;          // groups of CTAs on the symmetric tiles
     size_t sell_smem_ = 0;
     size_t solo_gmax_ = 1;       // groups the tables and barriers have room for
     int solo_nl_ = 0;            // lanes (the tables' first part)

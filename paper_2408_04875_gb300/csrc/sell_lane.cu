@@ -14,15 +14,10 @@
 //   * the rows a CTA owns live in registers of the warp that finishes them (x_{k-1}, g_{k-1},
 //     d - p, d + b'; for the eigen-solver its six vectors), x_k and g_k of every row in shared
 //     memory;
-//   * CTAs exchange a step's results in one hop instead of through a barrier, a record array
-//     and the vectors: a slice's 32 gradient entries and its partial sums are 64-bit pairs of a
-//     value and the step's tag, two to a 16-byte word; every CTA polls the words themselves until
-//     all their pairs carry the step's tag.  A pair is read and written whole, so nothing is
-//     fenced and nobody counts arrivals.  (Three values and one tag in a 128-bit access would be
-//     a third less to read, but the halves of such a word were seen to arrive one after the
-//     other: a record with the step's tag and the previous value.)  Words alternate between
-//     two buffers by the step's parity: a CTA stores the words of step j + 2 only after it has
-//     received all of step j + 1, and a CTA sends those only after it has read all of step j;
+//   * CTAs exchange a step's results in one hop, a slice's 32 gradient entries and its partial sums
+//     as tagged words (lane_words.cuh).  Words alternate between two buffers by the step's parity: a
+//     CTA stores the words of step j + 2 only after it has received all of step j + 1, and a CTA
+//     sends those only after it has read all of step j;
 //   * the scalar step (KKT test, BB step) is taken by every thread from the reduced sums,
 //     without a round through one thread and shared memory.
 //
@@ -40,7 +35,7 @@
 //
 // Lane vectors written by one CTA are read by others within the launch: plain loads of this
 // file are cached in L2 only (-dlcm=cg).
-#include "solo_common.cuh"
+#include "lane_words.cuh"
 
 namespace ubqp {
 
@@ -49,74 +44,7 @@ namespace {
 constexpr int kRowWords = 16;                 // 32 values, two to a word
 constexpr int kRecWords = 5;                  // the ten numbers of an Alg. 2 record
 constexpr int kStepWords = kRowWords + kRecWords;
-// the eigen-solver's twelve Gram sums (a word each): products of the row vectors x, Ax, w, Aw, p, Ap
-// (0 .. 5) in row_epilogue's order, sum t in nibble t
-constexpr int kGramWords = 12;
-constexpr unsigned long long kGramLeft = 0x422000422000ull, kGramRight = 0x442420553531ull;
 static_assert(kGramWords <= kStepWords && kSellWordsPerBlock == 2 * (kStepWords + kRowWords), "exchange words per block");
-
-// warp-level result of a reduction: the sums and maxima of one phase
-struct WarpRed {
-    float2 s[12];
-    float m[4];
-};
-
-// two values, each with the tag in its own 64 bits (the unit that is read and written whole)
-__device__ __forceinline__ void st_word(ulonglong2* p, float a, float b, uint32_t tag)
-{
-    const unsigned long long t = (unsigned long long)tag << 32;
-    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(t | __float_as_uint(a)),
-                 "l"(t | __float_as_uint(b))
-                 : "memory");
-}
-
-// one warp stores a slice's words, lane t word t; the warp is whole again before it waits
-__device__ __forceinline__ void publish(ulonglong2* p, bool mine, int lane, float2 v, uint32_t tag)
-{
-    if (mine) st_word(p + lane, v.x, v.y, tag);
-    __syncwarp();
-}
-
-__device__ __forceinline__ ulonglong2 ld_word(const ulonglong2* p)
-{
-    ulonglong2 v;
-    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ bool has_tag(ulonglong2 v, uint32_t tag)
-{
-    return (uint32_t)(v.x >> 32) == tag && (uint32_t)(v.y >> 32) == tag;
-}
-__device__ __forceinline__ float2 word_values(ulonglong2 v)
-{
-    return make_float2(__uint_as_float((uint32_t)v.x), __uint_as_float((uint32_t)v.y));
-}
-
-// Waits until the N words p[h] of every thread of the warp carry `tag` (threads without words of
-// their own pass another's).  The warp leaves the loop as a whole: with a loop that each thread
-// left by itself, the threads still waiting ran one after another, a trip to L2 each (20,000
-// cycles a wait with 16 of them, against 1,700).
-template <int N>
-__device__ __forceinline__ void wait_words(const SoloArgs& A, const ulonglong2* const (&p)[N], uint32_t tag,
-                                           ulonglong2 (&v)[N], volatile int* s_ok)
-{
-    const long long t0 = clock64();
-    for (;;) {
-#pragma unroll
-        for (int h = 0; h < N; ++h) v[h] = ld_word(p[h]);
-        bool all = true;
-#pragma unroll
-        for (int h = 0; h < N; ++h) all &= has_tag(v[h], tag);
-        if (__all_sync(0xffffffffu, all)) return;
-        const bool late = clock64() - t0 > (long long)A.wait_cycles || !*s_ok;
-        if (__any_sync(0xffffffffu, late)) {
-            atomicExch(A.err, 1);
-            *s_ok = 0;
-            return;
-        }
-    }
-}
 
 // sum of the shared-memory copy of one share (cnt entries of a slice, thread = row): groups of four
 // products as FMA chains, added to a compensated sum, the up to seven entries left over one by
@@ -207,31 +135,6 @@ __device__ __forceinline__ float2 share_gmem(const float* V, const uint16_t* C, 
     return acc;
 }
 
-// the butterfly of N compensated sums and M maxima, level by level (acc_shfl_reduce's order)
-template <int N, int M>
-__device__ __forceinline__ void butterfly(float2* s, float* m)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        float2 w[N > 0 ? N : 1];
-        float wm[M > 0 ? M : 1];
-#pragma unroll
-        for (int t = 0; t < N; ++t) {
-            w[t].x = __shfl_xor_sync(0xffffffffu, s[t].x, o);
-            w[t].y = __shfl_xor_sync(0xffffffffu, s[t].y, o);
-        }
-#pragma unroll
-        for (int t = 0; t < M; ++t) wm[t] = __shfl_xor_sync(0xffffffffu, m[t], o);
-#pragma unroll
-        for (int t = 0; t < N; ++t) s[t] = csum_merge(s[t], w[t]);
-#pragma unroll
-        for (int t = 0; t < M; ++t) m[t] = fmaxf(m[t], wm[t]);
-    }
-}
-
-// where g_{k-1} of a subproblem stopped before step k is kept (solo.cu alternates the two)
-__device__ __forceinline__ int g_buf(int k) { return (k & 1) ? V_G : V_W; }
-
 // the slices of a lane that this CTA owns: rank, rank + nc, ... (`one`: every slice of a lane of
 // one block, the CTA's warps shared out over them)
 struct Slices {
@@ -249,37 +152,6 @@ struct SliceAt {
 struct __align__(16) ShareAt {
     int k0, cnt, v, c;
 };
-
-// two of the 32 values held one per lane, for the word `lane` of a slice's row words
-__device__ __forceinline__ float2 row_word(float g, int lane)
-{
-    const float a = __shfl_sync(0xffffffffu, g, (2 * lane) & 31);
-    return make_float2(a, __shfl_sync(0xffffffffu, g, (2 * lane + 1) & 31));
-}
-
-// every slice's row words of buffer w (stride words per slice) into dst (32 values per slice)
-// (threads tid of nt, whole warps)
-__device__ __forceinline__ void gather_rows(const SoloArgs& A, const ulonglong2* w, int stride, int nblk, uint32_t tag,
-                                            float* dst, int tid, int nt, volatile int* s_ok)
-{
-    constexpr int kFly = 8;
-    const int nq = kRowWords * nblk;
-    for (int base = tid & ~31; base < nq; base += kFly * nt) {
-        const int q0 = base + (tid & 31);
-        const ulonglong2* p[kFly];
-        ulonglong2 v[kFly];
-#pragma unroll
-        for (int h = 0; h < kFly; ++h) {
-            int q = q0 + h * nt;
-            if (q >= nq) q = min(q0, nq - 1);
-            p[h] = w + (size_t)(q / kRowWords) * stride + q % kRowWords;
-        }
-        wait_words<kFly>(A, p, tag, v, s_ok);
-#pragma unroll
-        for (int h = 0; h < kFly; ++h)
-            if (q0 + h * nt < nq) reinterpret_cast<float2*>(dst)[q0 + h * nt] = word_values(v[h]);
-    }
-}
 
 }  // namespace
 
@@ -576,7 +448,7 @@ __global__ void __launch_bounds__(kThreads, kPer) sell_lane_kernel(SoloArgs A)
                             }
                         }
                         if (nc > 1 && warp >= gw0)
-                            gather_rows(A, w, kStepWords, nblk, tag, sg, tid - 32 * gw0, kThreads - 32 * gw0, &s_ok);
+                            gather_rows<kRowWords>(A, w, kStepWords, nblk, tag, sg, tid - 32 * gw0, kThreads - 32 * gw0, &s_ok);
                         __syncthreads();
                     }
                     if (!s_ok) break;
@@ -790,7 +662,7 @@ __global__ void __launch_bounds__(kThreads, kPer) sell_lane_kernel(SoloArgs A)
                             const float2 p = row_word(u, lane);
                             publish(wu + (size_t)sl.at(warp) * kRowWords, lane < kRowWords, lane, p, tag + 1u);
                         }
-                        gather_rows(A, wu, kRowWords, nblk, tag + 1u, su, tid, kThreads, &s_ok);
+                        gather_rows<kRowWords>(A, wu, kRowWords, nblk, tag + 1u, su, tid, kThreads, &s_ok);
                     }
                     if (tid == 0) S.updates += 1;
                     ++upd;

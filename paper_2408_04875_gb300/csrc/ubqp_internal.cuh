@@ -128,8 +128,8 @@ struct LaneDev {
     const float* spv;
     const uint16_t* spc;
     const int64_t* spo;
-    ulonglong2* xch;       // sliced lanes on groups of CTAs: the exchange words (kSellWordsPerBlock
-                           // per row block, zeroed before the first launch), else null
+    ulonglong2* xch;       // lanes on groups of CTAs (sell_lane.cu, sym_lane.cu): the exchange words,
+                           // zeroed before the first launch, else null
 };
 
 // solver constants (kernel parameter)
@@ -500,7 +500,8 @@ struct SoloArgs {
                                 // takes longer than the wait it would bound
     int32_t fast;               // Alg. 2 steps with one barrier (whole x_k in every CTA)
     int32_t one_ok;             // shared memory holds the one-CTA state (6 vectors)
-    int32_t mat_bytes;          // sell_lane.cu: shared memory of a CTA for its slices' entries
+    int32_t mat_bytes;          // sell_lane.cu, sym_lane.cu: shared memory of a CTA for its entries / tiles
+    const SymLane* sym;         // sym_lane.cu: per lane
     Params P;
 };
 constexpr int kSoloBarStride = 32;   // unsigned per group barrier (128 bytes)
@@ -517,6 +518,12 @@ constexpr int kSellWordsPerBlock = 74;   // 16-byte exchange words per row block
 size_t sell_smem_limit(int per);
 bool sell_fits(int per, size_t smem);
 cudaError_t launch_sell(const SoloArgs& a, int per, size_t smem, cudaStream_t s);
+
+// the same groups on the symmetric tiles, at most kSymMaxTiles tiles per CTA (sym_lane.cu)
+constexpr int kSymMaxTiles = 20;
+size_t sym_lane_words(int nb);
+size_t sym_lane_smem(int ld, int tiles, int32_t* mat_bytes);
+cudaError_t launch_sym(const SoloArgs& a, size_t smem, cudaStream_t s);
 
 cudaError_t prepare_lane_loop(int max_ld);
 int lane_loop_grid(int max_ld);
