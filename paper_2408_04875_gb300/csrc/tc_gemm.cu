@@ -141,6 +141,21 @@ __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint6
         : "memory");
 }
 
+// Position in a ring of ns slots: slot and how often the ring has been round (its parity is what the
+// barriers want).  Kept by increments: dividing a running count by ns, and the k-step by the number
+// of chains below, cost the one issuing thread 680 cycles a k-block, twice what its copies took.
+struct RingPos {
+    int s;
+    uint32_t par;
+    __device__ __forceinline__ void next(int ns)
+    {
+        if (++s == ns) {
+            s = 0;
+            par ^= 1u;
+        }
+    }
+};
+
 __device__ __forceinline__ void umma_commit(uint64_t* bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
@@ -171,6 +186,17 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v)
 // column, the hi parts of the chains in ascending order, then the lo parts; both kernels use
 // this layout, so a tile's sums do not depend on which kernel computed it.
 __host__ __device__ constexpr int tc_chains_k(int bn) { return bn <= 32 ? 4 : (bn <= 64 ? 2 : 1); }
+
+// the four K-steps of one k-block; k-step ks of a tile goes to chain ks % nk, nk = 1, 2 or 4, so
+// step k of any k-block to chain k % nk, and each chain's first step starts its accumulator
+__device__ __forceinline__ void umma_kblock(uint32_t d, uint32_t sa, uint32_t sb, uint32_t idesc, int nk, uint32_t w,
+                                            bool first)
+{
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        umma_bf16(d + (uint32_t)(k & (nk - 1)) * w, sdesc_sw128(sa + k * 32), sdesc_sw128(sb + k * 32), idesc,
+                  first && k < nk ? 0u : 1u);
+}
 
 // 16 consecutive output columns of this thread's TMEM lane, summed over terms and chains
 __device__ __forceinline__ void tmem_ld16_sum(uint32_t taddr, int bn, bool two, float* v)
@@ -487,9 +513,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) phase_a_tc_kernel(TcArgs A)
         if (warp == 0 && lane == 0) {
             // TMA producer
             int issued = 0;
-            for (int kb = 0; kb < nkb; ++kb) {
-                const int s = kb % NS;
-                if (kb >= NS && !mbar_wait(&empty_bar[s], (uint32_t)((kb / NS - 1) & 1))) { s_fail = 1; break; }
+            RingPos q{0, 1u};   // the first round finds every slot empty
+            for (int kb = 0; kb < nkb; ++kb, q.next(NS)) {
+                const int s = q.s;
+                if (kb >= NS && !mbar_wait(&empty_bar[s], q.par)) { s_fail = 1; break; }
                 issued = kb + 1;
                 unsigned char* st = ring + (size_t)s * stage_bytes;
                 mbar_expect_tx(&full_bar[s], stage_bytes);
@@ -506,19 +533,15 @@ __global__ void __launch_bounds__(kTcThreads, 1) phase_a_tc_kernel(TcArgs A)
         } else if (warp == 1 && lane == 0) {
             // MMA issuer: 4 K-steps of 16 per 64-wide k-block, both terms in one MMA of N = 2 BN
             const uint32_t idesc = idesc_bf16(128, two ? 2 * BN : BN);
-            const int NK = tc_chains_k(BN), W = two ? 2 * BN : BN;
-            for (int kb = 0; kb < nkb; ++kb) {
-                const int s = kb % NS;
-                if (!mbar_wait(&full_bar[s], (uint32_t)((kb / NS) & 1))) { s_fail = 1; break; }
+            const int NK = tc_chains_k(BN);
+            const uint32_t W = (uint32_t)(two ? 2 * BN : BN);
+            RingPos q{0, 0u};
+            for (int kb = 0; kb < nkb; ++kb, q.next(NS)) {
+                const int s = q.s;
+                if (!mbar_wait(&full_bar[s], q.par)) { s_fail = 1; break; }
                 tc_fence_after();
                 const uint32_t sa = smem_u32(ring + (size_t)s * stage_bytes);
-                const uint32_t sb = sa + a_bytes;
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int ks = kb * 4 + k, ck = ks % NK;
-                    umma_bf16(tmem + (uint32_t)(ck * W), sdesc_sw128(sa + k * 32), sdesc_sw128(sb + k * 32), idesc,
-                              ks >= NK ? 1u : 0u);
-                }
+                umma_kblock(tmem, sa, sa + a_bytes, idesc, NK, W, kb == 0);
                 umma_commit(&empty_bar[s]);
             }
             umma_commit(&accum_bar);
@@ -746,6 +769,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) phase_a_tcp_kernel(TcArgs A, in
     if (warp == 0) {
         if (lane == 0) {   // ---- TMA producer
             long long pos = 0;
+            RingPos q{0, 1u};   // the first round finds every slot empty
             for (int t = blockIdx.x; t < ntiles && !vload(&s_fail); t += gridDim.x) {
                 const TcTile T = tcp_tile(A, t);
                 if (!T.alive) continue;
@@ -753,10 +777,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) phase_a_tcp_kernel(TcArgs A, in
                 const bool two = I.two_terms != 0;
                 const uint32_t a_bytes = 128u * 128u, b_bytes = (uint32_t)I.bn * 128u;
                 const uint32_t sb = a_bytes + b_bytes * (two ? 2u : 1u);
-                for (int kb = 0; kb < T.kb; ++kb, ++pos) {
-                    const int s = (int)(pos % NS);
-                    const long long use = pos / NS;
-                    if (use > 0 && !mbar_wait(&empty_bar[s], (uint32_t)((use - 1) & 1))) {
+                for (int kb = 0; kb < T.kb; ++kb, ++pos, q.next(NS)) {
+                    const int s = q.s;
+                    if (pos >= NS && !mbar_wait(&empty_bar[s], q.par)) {
                         s_fail = 1;
                         break;
                     }
@@ -772,6 +795,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) phase_a_tcp_kernel(TcArgs A, in
     } else if (warp == 1) {
         if (lane == 0) {   // ---- MMA issuer
             long long pos = 0;
+            RingPos q{0, 0u};
             int j = 0;
             for (int t = blockIdx.x; t < ntiles && !vload(&s_fail); t += gridDim.x) {
                 const TcTile T = tcp_tile(A, t);
@@ -787,23 +811,18 @@ __global__ void __launch_bounds__(kTcThreads, 1) phase_a_tcp_kernel(TcArgs A, in
                 tc_fence_after();
                 const uint32_t d = tmem + (uint32_t)buf * col_stride;
                 const uint32_t idesc = idesc_bf16(128, two ? 2 * I.bn : I.bn);
-                const int NK = tc_chains_k(I.bn), W = two ? 2 * I.bn : I.bn;
+                const int NK = tc_chains_k(I.bn);
+                const uint32_t W = (uint32_t)(two ? 2 * I.bn : I.bn);
                 bool ok = true;
-                for (int kb = 0; kb < T.kb; ++kb, ++pos) {
-                    const int s = (int)(pos % NS);
-                    if (!mbar_wait(&full_bar[s], (uint32_t)((pos / NS) & 1))) {
+                for (int kb = 0; kb < T.kb; ++kb, ++pos, q.next(NS)) {
+                    const int s = q.s;
+                    if (!mbar_wait(&full_bar[s], q.par)) {
                         ok = false;
                         break;
                     }
                     tc_fence_after();
                     const uint32_t sa = smem_u32(ring + (size_t)s * stage_max);
-                    const uint32_t sbh = sa + a_bytes;
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const int ks = kb * 4 + k, ck = ks % NK;
-                        umma_bf16(d + (uint32_t)(ck * W), sdesc_sw128(sa + k * 32), sdesc_sw128(sbh + k * 32), idesc,
-                                  ks >= NK ? 1u : 0u);
-                    }
+                    umma_kblock(d, sa, sa + a_bytes, idesc, NK, W, kb == 0);
                     umma_commit(&empty_bar[s]);
                 }
                 if (!ok) {
