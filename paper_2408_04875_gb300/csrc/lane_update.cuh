@@ -66,163 +66,175 @@ __host__ __device__ __forceinline__ float rr_rsqrt(float v)
 #endif
 }
 
-// smallest eigenpair of a symmetric k x k matrix (k <= 3) by cyclic Jacobi rotations.
+// a b + c rounded once, and a b never fused into what follows (the host form for the tests)
+__host__ __device__ __forceinline__ float rr_fma(float a, float b, float c)
+{
+#ifdef __CUDA_ARCH__
+    return __fmaf_rn(a, b, c);
+#else
+    return fmaf(a, b, c);
+#endif
+}
+__host__ __device__ __forceinline__ float rr_mul(float a, float b)
+{
+#ifdef __CUDA_ARCH__
+    return __fmul_rn(a, b);
+#else
+    return a * b;
+#endif
+}
+
+// smallest eigenpair of a symmetric K x K matrix (K <= 3) by cyclic Jacobi rotations.
 // FP32 throughout: FP64 runs at a small fraction of the FP32 rate on this part, and the
-// preconditioned basis keeps the 3 x 3 Gram matrices well scaled.  Every loop runs over the
-// full 3 x 3 with the entries outside k x k masked, so that all indices are compile-time
-// constants and the matrices stay in registers (the operations and their order are those
-// of the k x k loops).
-__host__ __device__ __forceinline__ void small_sym_eig_min(int k, float (&M)[3][3], float& lam, float (&v)[3])
+// preconditioned basis keeps the 3 x 3 Gram matrices well scaled.  K is a compile-time constant:
+// the matrices stay in registers and no index or mask is computed (one thread runs this, so its
+// latency is the step's: 6,600 cycles of the eigen-solver's decision with run-time k).  Where a
+// product is fused into a sum is written out, so that every kernel this is compiled into, and any
+// unrolling, gives the same bits.
+template <int K>
+__host__ __device__ __forceinline__ void sym_eig_min(float (&M)[3][3], float& lam, float (&v)[3])
 {
     float V[3][3] = {{1.f, 0.f, 0.f}, {0.f, 1.f, 0.f}, {0.f, 0.f, 1.f}};
+#pragma unroll 1
     for (int sweep = 0; sweep < 8; ++sweep) {
         float off = 0.f, dia = 0.f;
 #pragma unroll
-        for (int p = 0; p < 3; ++p) {
-            if (p >= k) break;
-            dia += M[p][p] * M[p][p];
+        for (int p = 0; p < K; ++p) {
+            dia = rr_fma(M[p][p], M[p][p], dia);
 #pragma unroll
-            for (int q = p + 1; q < 3; ++q)
-                if (q < k) off += M[p][q] * M[p][q];
+            for (int q = p + 1; q < K; ++q) off = rr_fma(M[p][q], M[p][q], off);
         }
         if (off <= 1e-14f * dia) break;
 #pragma unroll
-        for (int p = 0; p < 3; ++p)
+        for (int p = 0; p < K; ++p)
 #pragma unroll
-            for (int q = p + 1; q < 3; ++q) {
-                if (q >= k || M[p][q] == 0.f) continue;
+            for (int q = p + 1; q < K; ++q) {
+                if (M[p][q] == 0.f) continue;
                 float theta = (M[q][q] - M[p][p]) / (2.f * M[p][q]);
-                float t = (theta >= 0.f ? 1.f : -1.f) / (fabsf(theta) + sqrtf(theta * theta + 1.f));
-                float c = rr_rsqrt(t * t + 1.f), sn = t * c;
+                float t = (theta >= 0.f ? 1.f : -1.f) / (fabsf(theta) + sqrtf(rr_fma(theta, theta, 1.f)));
+                float c = rr_rsqrt(rr_fma(t, t, 1.f)), sn = rr_mul(t, c);
 #pragma unroll
-                for (int r = 0; r < 3; ++r) {
-                    if (r >= k) break;
+                for (int r = 0; r < K; ++r) {
                     float mrp = M[r][p], mrq = M[r][q];
-                    M[r][p] = c * mrp - sn * mrq;
-                    M[r][q] = sn * mrp + c * mrq;
+                    M[r][p] = rr_fma(c, mrp, -rr_mul(sn, mrq));
+                    M[r][q] = rr_fma(sn, mrp, rr_mul(c, mrq));
                 }
 #pragma unroll
-                for (int r = 0; r < 3; ++r) {
-                    if (r >= k) break;
+                for (int r = 0; r < K; ++r) {
                     float mpr = M[p][r], mqr = M[q][r];
-                    M[p][r] = c * mpr - sn * mqr;
-                    M[q][r] = sn * mpr + c * mqr;
+                    M[p][r] = rr_fma(c, mpr, -rr_mul(sn, mqr));
+                    M[q][r] = rr_fma(sn, mpr, rr_mul(c, mqr));
                 }
 #pragma unroll
-                for (int r = 0; r < 3; ++r) {
-                    if (r >= k) break;
+                for (int r = 0; r < K; ++r) {
                     float vrp = V[r][p], vrq = V[r][q];
-                    V[r][p] = c * vrp - sn * vrq;
-                    V[r][q] = sn * vrp + c * vrq;
+                    V[r][p] = rr_fma(c, vrp, -rr_mul(sn, vrq));
+                    V[r][q] = rr_fma(sn, vrp, rr_mul(c, vrq));
                 }
             }
     }
     int j = 0;
     lam = M[0][0];
-    if (k > 1 && M[1][1] < lam) { j = 1; lam = M[1][1]; }
-    if (k > 2 && M[2][2] < lam) { j = 2; lam = M[2][2]; }
+    if (K > 1 && M[1][1] < lam) { j = 1; lam = M[1][1]; }
+    if (K > 2 && M[2][2] < lam) { j = 2; lam = M[2][2]; }
 #pragma unroll
-    for (int r = 0; r < 3; ++r) v[r] = r < k ? (j == 0 ? V[r][0] : (j == 1 ? V[r][1] : V[r][2])) : 0.f;
+    for (int r = 0; r < 3; ++r) v[r] = r < K ? (j == 0 ? V[r][0] : (j == 1 ? V[r][1] : V[r][2])) : 0.f;
+}
+
+__host__ __device__ __forceinline__ void small_sym_eig_min(int k, float (&M)[3][3], float& lam, float (&v)[3])
+{
+    if (k == 3) sym_eig_min<3>(M, lam, v);
+    else if (k == 2) sym_eig_min<2>(M, lam, v);
+    else sym_eig_min<1>(M, lam, v);
+}
+
+// Rayleigh-Ritz on the first K directions of span{x, w, p}, FP32: 1 done, 0 a value that is not
+// finite, -1 a direction without length or a nearly dependent basis
+template <int K>
+__host__ __device__ __forceinline__ int rr_step(const float (&A)[3][3], const float (&B)[3][3], float& lam, float (&c)[3])
+{
+    float sc[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int t = 0; t < K; ++t) {
+        if (!(B[t][t] > 0.f)) return -1;
+        sc[t] = rr_rsqrt(B[t][t]);
+    }
+    float As[3][3], Bs[3][3];
+#pragma unroll
+    for (int r = 0; r < K; ++r)
+#pragma unroll
+        for (int q = 0; q < K; ++q) {
+            As[r][q] = A[r][q] * sc[r] * sc[q];
+            Bs[r][q] = B[r][q] * sc[r] * sc[q];
+        }
+    // Cholesky Bs = L L^T; a pivot below 1e-3 (unit diagonal) means a nearly dependent
+    // basis in FP32: drop the last direction and retry
+    float Lc[3][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
+#pragma unroll
+    for (int j = 0; j < K; ++j) {
+        float sd = Bs[j][j];
+#pragma unroll
+        for (int t = 0; t < j; ++t) sd = rr_fma(-Lc[j][t], Lc[j][t], sd);
+        if (!(sd > 1e-3f)) return -1;
+        Lc[j][j] = sqrtf(sd);
+#pragma unroll
+        for (int i = j + 1; i < K; ++i) {
+            float u = Bs[i][j];
+#pragma unroll
+            for (int t = 0; t < j; ++t) u = rr_fma(-Lc[i][t], Lc[j][t], u);
+            Lc[i][j] = u / Lc[j][j];
+        }
+    }
+    float Li[3][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
+#pragma unroll
+    for (int j = 0; j < K; ++j) {
+        Li[j][j] = 1.f / Lc[j][j];
+#pragma unroll
+        for (int i = j + 1; i < K; ++i) {
+            float u = 0.f;
+#pragma unroll
+            for (int t = j; t < i; ++t) u = rr_fma(-Lc[i][t], Li[t][j], u);
+            Li[i][j] = u / Lc[i][i];
+        }
+    }
+    float M[3][3];
+#pragma unroll
+    for (int r = 0; r < K; ++r)
+#pragma unroll
+        for (int q = 0; q < K; ++q) {
+            float u = 0.f;
+#pragma unroll
+            for (int a = 0; a < K; ++a)
+#pragma unroll
+                for (int b = 0; b < K; ++b) u = rr_fma(rr_mul(Li[r][a], As[a][b]), Li[q][b], u);
+            M[r][q] = u;
+        }
+    float v[3];
+    sym_eig_min<K>(M, lam, v);
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {  // c = sc * L^-T v
+        float u = 0.f;
+        if (r < K)
+#pragma unroll
+            for (int a = r; a < K; ++a) u = rr_fma(Li[a][r], v[a], u);
+        c[r] = r < K ? u * sc[r] : 0.f;
+    }
+    return isfinite(lam) ? 1 : 0;
 }
 
 // Rayleigh-Ritz on span{x, w, p} (p only when has_p), FP32.  Returns false on breakdown.
 // Gram entries: ga = (xAx, xAw, xAp, wAw, wAp, pAp), gb = (xx, xw, xp, ww, wp, pp).
-// Loops as in small_sym_eig_min: full 3 x 3, masked to k x k.  Not inlined: its registers are
-// needed only for the eigen-solver's decision, not in the kernels' hot loops.
+// A nearly dependent p is dropped.  Not inlined: its registers are needed only for the
+// eigen-solver's decision, not in the kernels' hot loops.
 static __host__ __device__ __noinline__ bool rayleigh_ritz(const float (&ga)[6], const float (&gb)[6], bool has_p, float& lam,
                                               float (&c)[3])
 {
     const float A[3][3] = {{ga[0], ga[1], ga[2]}, {ga[1], ga[3], ga[4]}, {ga[2], ga[4], ga[5]}};
     const float B[3][3] = {{gb[0], gb[1], gb[2]}, {gb[1], gb[3], gb[4]}, {gb[2], gb[4], gb[5]}};
-    int k = has_p ? 3 : 2;
     if (!(B[0][0] > 0.f)) return false;
-    for (int attempt = 0; attempt < 2; ++attempt) {
-        if (k < 2) return false;
-        float sc[3] = {0.f, 0.f, 0.f};
-        bool bad = false;
-#pragma unroll
-        for (int t = 0; t < 3; ++t) {
-            if (t >= k) break;
-            if (!(B[t][t] > 0.f)) { bad = true; break; }
-            sc[t] = rr_rsqrt(B[t][t]);
-        }
-        if (bad) { k -= 1; continue; }
-        float As[3][3], Bs[3][3];
-#pragma unroll
-        for (int r = 0; r < 3; ++r)
-#pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                As[r][q] = (r < k && q < k) ? A[r][q] * sc[r] * sc[q] : 0.f;
-                Bs[r][q] = (r < k && q < k) ? B[r][q] * sc[r] * sc[q] : 0.f;
-            }
-        // Cholesky Bs = L L^T; a pivot below 1e-3 (unit diagonal) means a nearly dependent
-        // basis in FP32: drop the last direction and retry
-        float Lc[3][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            if (j >= k || bad) break;
-            float sd = Bs[j][j];
-#pragma unroll
-            for (int t = 0; t < j; ++t) sd -= Lc[j][t] * Lc[j][t];
-            if (!(sd > 1e-3f)) { bad = true; break; }
-            Lc[j][j] = sqrtf(sd);
-#pragma unroll
-            for (int i = j + 1; i < 3; ++i) {
-                if (i >= k) break;
-                float u = Bs[i][j];
-#pragma unroll
-                for (int t = 0; t < j; ++t) u -= Lc[i][t] * Lc[j][t];
-                Lc[i][j] = u / Lc[j][j];
-            }
-        }
-        if (bad) { k -= 1; continue; }
-        float Li[3][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            if (j >= k) break;
-            Li[j][j] = 1.f / Lc[j][j];
-#pragma unroll
-            for (int i = j + 1; i < 3; ++i) {
-                if (i >= k) break;
-                float u = 0.f;
-#pragma unroll
-                for (int t = j; t < i; ++t) u -= Lc[i][t] * Li[t][j];
-                Li[i][j] = u / Lc[i][i];
-            }
-        }
-        float M[3][3];
-#pragma unroll
-        for (int r = 0; r < 3; ++r)
-#pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                float u = 0.f;
-                if (r < k && q < k)
-#pragma unroll
-                    for (int a = 0; a < 3; ++a) {
-                        if (a >= k) break;
-#pragma unroll
-                        for (int b = 0; b < 3; ++b) {
-                            if (b >= k) break;
-                            u += Li[r][a] * As[a][b] * Li[q][b];
-                        }
-                    }
-                M[r][q] = u;
-            }
-        float v[3];
-        small_sym_eig_min(k, M, lam, v);
-#pragma unroll
-        for (int r = 0; r < 3; ++r) {  // c = sc * L^-T v
-            float u = 0.f;
-#pragma unroll
-            for (int a = r; a < 3; ++a) {
-                if (a >= k) break;
-                u += Li[a][r] * v[a];
-            }
-            c[r] = r < k ? u * sc[r] : 0.f;
-        }
-        return isfinite(lam);
-    }
-    return false;
+    int rc = has_p ? rr_step<3>(A, B, lam, c) : -1;
+    if (rc < 0) rc = rr_step<2>(A, B, lam, c);
+    return rc > 0;
 }
 
 __device__ __forceinline__ float csum_value(float2 v) { return v.x + v.y; }
