@@ -123,24 +123,11 @@ __device__ __forceinline__ void reformulate_row(const RefArgs& a, int i)
     const int n = a.n, ld = a.ld;
     const double* Qrow = a.Q + (size_t)i * n;
     const double bi = a.b ? a.b[i] : 0.0;
-    // perturbed row and its absolute sum
-    double r = 0.0;
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        double q = Qrow[j];
-        double m = 0.0;
-        bool touch = (j == i) || (!a.diag_only_mu);
-        if (touch) {
-            if (a.mu) m = a.mu[(size_t)i * n + j];
-            else if (a.sigma > 0.0 && (q != 0.0 || j == i))
-                m = a.sigma * normal_draw(a.seed, (uint64_t)a.inst, (uint64_t)min(i, j), (uint64_t)max(i, j));
-        }
-        double qm = q + m;
-        r += fabs(qm);
-    }
-    r = block_sum_d<256>(r, shd);
-    const double gam = a.no_gamma ? 0.0 : 2.0 * r + fabs(bi) + a.margin;  // Eq. (gamma), strict ">"
-    // second pass: store Q'_off in the working precision and the off-diagonal row sum
-    double oabs = 0.0, dii = 0.0;
+    // One pass over the row: its absolute sum for gamma, Q'_off in the working precision with its
+    // row sum, and the evaluation matrix.  Only the diagonal waits for gamma.  (The perturbation's
+    // normal draws, two logarithms' worth of FP64 per stored entry, are what bounds this kernel: a
+    // second pass for the stored values drew them all again, 1.62 ms of a solve of n = 2500.)
+    double r = 0.0, oabs = 0.0, dii = 0.0;
     float offmax = 0.f;
     for (int j = threadIdx.x; j < ld; j += blockDim.x) {
         double q = j < n ? Qrow[j] : 0.0;
@@ -152,8 +139,9 @@ __device__ __forceinline__ void reformulate_row(const RefArgs& a, int i)
                 m = a.sigma * normal_draw(a.seed, (uint64_t)a.inst, (uint64_t)min(i, j), (uint64_t)max(i, j));
         }
         double qm = q + m;
+        if (j < n) r += fabs(qm);
         if (j == i) {
-            dii = qm + gam;
+            dii = qm;
             if (a.Qoff) a.Qoff[(size_t)i * ld + j] = 0.f;
             if (a.Qbf) a.Qbf[qbf_index(i, j, ld)] = __float2bfloat16_rn(0.f);
         } else {
@@ -176,6 +164,9 @@ __device__ __forceinline__ void reformulate_row(const RefArgs& a, int i)
             a.Qeval[(size_t)i * ld + j] = make_float2(hi, (float)(q - (double)hi));
         }
     }
+    r = block_sum_d<256>(r, shd);
+    const double gam = a.no_gamma ? 0.0 : 2.0 * r + fabs(bi) + a.margin;  // Eq. (gamma), strict ">"
+    dii += gam;
     oabs = block_sum_d<256>(oabs, shd);
     offmax = block_max<256>(offmax, shf);
     // dii was set by exactly one thread; share it
