@@ -853,6 +853,7 @@ class Solver {
                 const void* ub = ar_.at<char>(I.o_Uhi);
                 const void* lb = I.o_Ulo ? (const void*)ar_.at<char>(I.o_Ulo) : ub;
                 if (tc_encode_map(&h.tmA, ar_.at<char>(I.o_Qbf), (int64_t)I.ld * I.ld / 64, 64, 128) != CUDA_SUCCESS ||
+                    tc_encode_map(&h.tmA2, ar_.at<char>(I.o_Qbf), (int64_t)I.ld * I.ld / 64, 64, 256) != CUDA_SUCCESS ||
                     tc_encode_map(&h.tmBhi, ub, I.rows_b, I.ld, I.bn) != CUDA_SUCCESS ||
                     tc_encode_map(&h.tmBlo, lb, I.rows_b, I.ld, I.bn) != CUDA_SUCCESS) {
                     set_error("cuTensorMapEncodeTiled failed for instance %zu", t);
@@ -956,6 +957,7 @@ class Solver {
                 if (S == 0) {
                     if (tcp_stages < 2) continue;
                     a.stages = tcp_stages;
+                    a.kbs = tcp_pick_kbs(max_bn_, two);
                     a.tmem_cols = tcp_tmem_cols(two);
                 } else {
                     if (S > 1 && kb_min / S < 2) break;
@@ -1068,6 +1070,7 @@ class Solver {
             tca.fuse = (max_ld_ / 128 <= 32 && o_.tc_fuse != 0) ? 1 : 0;
             if (tcp_) {
                 tca.tmem_cols = tcp_tmem_cols(o_.precision == UBQP_BF16X2_TC);
+                tca.kbs = tcp_pick_kbs(max_bn_, o_.precision == UBQP_BF16X2_TC);
                 tcp_grid_ = tcp_grid(tca, tc_tiles_);
             }
         }

@@ -34,6 +34,7 @@ namespace ubqp {
 
 namespace {
 
+constexpr int kTcpThreads = 288;      // persistent kernel: a ninth warp copies the inputs
 constexpr int kTcThreads = 256;       // 8 warps: TMA producer, MMA issuer, then all 8 drain TMEM / run the epilogue
 constexpr uint64_t kWaitNs = 2000000000ull;
 // split-K kernel epilogue: each warp stages the operand rows of its next kEpiDepth lanes in
@@ -85,6 +86,24 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity)
             : "memory");
         if (done) return true;
         if (globaltimer() - t0 > kWaitNs) return false;
+    }
+}
+
+// the same by a whole warp, which leaves together: true for all or, when any thread's limit ran out,
+// false for all
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity)
+{
+    const uint32_t addr = smem_u32(bar);
+    const uint64_t t0 = globaltimer();
+    for (;;) {
+        uint32_t done;
+        asm volatile(
+            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(done)
+            : "r"(addr), "r"(parity)
+            : "memory");
+        if (__all_sync(0xffffffffu, done != 0u)) return true;
+        if (__any_sync(0xffffffffu, globaltimer() - t0 > kWaitNs)) return false;
     }
 }
 
@@ -140,6 +159,17 @@ __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint6
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum)
         : "memory");
 }
+
+// One thread of a whole warp.  The producing and issuing warps walk their loops as whole warps and
+// only the copy, MMA and commit instructions are one thread's: with the loop itself in one thread's
+// branch, every operand of those instructions had to be moved to a uniform register first.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(p));
+    return p != 0u;
+}
+__device__ __forceinline__ uint32_t uniform(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
 
 // Position in a ring of ns slots: slot and how often the ring has been round (its parity is what the
 // barriers want).  Kept by increments: dividing a running count by ns, and the k-step by the number
@@ -510,41 +540,49 @@ __global__ void __launch_bounds__(kTcThreads, 1) phase_a_tc_kernel(TcArgs A)
 
     if (!s_skip && nkb > 0) {
         const uint32_t tmem = tmem_base;
-        if (warp == 0 && lane == 0) {
+        if (warp == 0) {
             // TMA producer
             int issued = 0;
+            const bool one = elect_one();
             RingPos q{0, 1u};   // the first round finds every slot empty
             for (int kb = 0; kb < nkb; ++kb, q.next(NS)) {
                 const int s = q.s;
-                if (kb >= NS && !mbar_wait(&empty_bar[s], q.par)) { s_fail = 1; break; }
+                if (kb >= NS && !mbar_wait_warp(&empty_bar[s], q.par)) { s_fail = 1; break; }
                 issued = kb + 1;
-                unsigned char* st = ring + (size_t)s * stage_bytes;
-                mbar_expect_tx(&full_bar[s], stage_bytes);
-                const int kx = (kb0 + kb) * 64;
-                tma_load_2d(st, &I.tmA, &full_bar[s], 0, (mt * kb_total + kb0 + kb) * 128);
-                tma_load_2d(st + a_bytes, &I.tmBhi, &full_bar[s], kx, nt * BN);
-                if (two) tma_load_2d(st + a_bytes + b_bytes, &I.tmBlo, &full_bar[s], kx, nt * BN);
+                if (one) {
+                    unsigned char* st = ring + (size_t)s * stage_bytes;
+                    mbar_expect_tx(&full_bar[s], stage_bytes);
+                    const int kx = (kb0 + kb) * 64;
+                    tma_load_2d(st, &I.tmA, &full_bar[s], 0, (mt * kb_total + kb0 + kb) * 128);
+                    tma_load_2d(st + a_bytes, &I.tmBhi, &full_bar[s], kx, nt * BN);
+                    if (two) tma_load_2d(st + a_bytes + b_bytes, &I.tmBlo, &full_bar[s], kx, nt * BN);
+                }
+                __syncwarp();
             }
             if (s_fail) {
                 // a wait ran out: let every copy already issued land before the ring is reused
                 for (int kb = (issued > NS ? issued - NS : 0); kb < issued; ++kb)
                     mbar_wait(&full_bar[kb % NS], (uint32_t)((kb / NS) & 1));
             }
-        } else if (warp == 1 && lane == 0) {
+        } else if (warp == 1) {
             // MMA issuer: 4 K-steps of 16 per 64-wide k-block, both terms in one MMA of N = 2 BN
             const uint32_t idesc = idesc_bf16(128, two ? 2 * BN : BN);
             const int NK = tc_chains_k(BN);
             const uint32_t W = (uint32_t)(two ? 2 * BN : BN);
+            const bool one = elect_one();
             RingPos q{0, 0u};
             for (int kb = 0; kb < nkb; ++kb, q.next(NS)) {
                 const int s = q.s;
-                if (!mbar_wait(&full_bar[s], q.par)) { s_fail = 1; break; }
+                if (!mbar_wait_warp(&full_bar[s], q.par)) { s_fail = 1; break; }
                 tc_fence_after();
-                const uint32_t sa = smem_u32(ring + (size_t)s * stage_bytes);
-                umma_kblock(tmem, sa, sa + a_bytes, idesc, NK, W, kb == 0);
-                umma_commit(&empty_bar[s]);
+                const uint32_t sa = uniform(smem_u32(ring + (size_t)s * stage_bytes));
+                if (one) {
+                    umma_kblock(tmem, sa, sa + a_bytes, idesc, NK, W, kb == 0);
+                    umma_commit(&empty_bar[s]);
+                }
+                __syncwarp();
             }
-            umma_commit(&accum_bar);
+            if (one) umma_commit(&accum_bar);
         }
         __syncwarp();
     }
@@ -684,8 +722,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) phase_a_tc_kernel(TcArgs A)
 // SM walks the tiles blockIdx.x, blockIdx.x + gridDim.x, ... and overlaps the epilogue of
 // one tile with the contraction of the next.
 //
-// Roles: warp 0 (one thread) keeps the TMA ring full across tile boundaries; warp 1 (one
-// thread) issues the MMAs of each tile into one of two TMEM accumulators (columns
+// Roles: warp 0 keeps the ring full of Q_off across tile boundaries and warp 8 of the starts'
+// inputs (a slot is two k-blocks: one copy of Q_off, two or four of inputs; with one producer and
+// one k-block per slot its instructions set the pace, 600 cycles a k-block); warp 1 issues the MMAs of each tile into one of two TMEM accumulators (columns
 // buf * max_bn), waiting until the epilogue has drained that buffer; warps 4..7 drain the
 // finished accumulator into shared memory (each warp reaches TMEM lanes 32 (w mod 4) ..)
 // and release it; warps 2..7 then run the per-row epilogue of the tile's lanes.  All roles
@@ -731,24 +770,25 @@ __device__ __forceinline__ void epi_bar_sync() { asm volatile("bar.sync 1, 192;"
 
 __device__ __forceinline__ int vload(const int* p) { return *reinterpret_cast<const volatile int*>(p); }
 
-__global__ void __launch_bounds__(kTcThreads, 1) phase_a_tcp_kernel(TcArgs A, int ntiles)
+__global__ void __launch_bounds__(kTcpThreads, 1) phase_a_tcp_kernel(TcArgs A, int ntiles)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* ring = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int NS = A.stages;
-    const uint32_t stage_max = 128u * 128u + (uint32_t)A.max_bn * 128u * (A.two_any ? 2u : 1u);
+    const int KB = A.kbs;   // every k-block count (ld / 64, ld a multiple of 128) is even
+    const uint32_t stage_max = (uint32_t)KB * (128u * 128u + (uint32_t)A.max_bn * 128u * (A.two_any ? 2u : 1u));
     float* P = reinterpret_cast<float*>(ring + (size_t)NS * stage_max);
     __shared__ uint64_t full_bar[kTcpMaxStages], empty_bar[kTcpMaxStages], accf_bar[2], acce_bar[2], fin_bar;
     __shared__ uint32_t tmem_base;
     __shared__ int s_fail;
-    __shared__ long long s_issued;
+    __shared__ long long s_issued[2];
     __shared__ WarpUpd s_upd[kTcThreads / 32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t col_stride = A.two_any ? 256u : 128u;   // one accumulator buffer: terms x chains x bn <= this
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < NS; ++s) {
-            mbar_init(&full_bar[s], 1);
+            mbar_init(&full_bar[s], 2);   // both producers
             mbar_init(&empty_bar[s], 1);
         }
         for (int b = 0; b < 2; ++b) {
@@ -758,7 +798,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) phase_a_tcp_kernel(TcArgs A, in
         mbar_init(&fin_bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         s_fail = 0;
-        s_issued = 0;
+        s_issued[0] = s_issued[1] = 0;
     }
     if (warp == 1) tmem_alloc(&tmem_base, (uint32_t)A.tmem_cols);
     tc_fence_before();
@@ -766,77 +806,91 @@ __global__ void __launch_bounds__(kTcThreads, 1) phase_a_tcp_kernel(TcArgs A, in
     tc_fence_after();
     const uint32_t tmem = tmem_base;
 
-    if (warp == 0) {
-        if (lane == 0) {   // ---- TMA producer
-            long long pos = 0;
-            RingPos q{0, 1u};   // the first round finds every slot empty
-            for (int t = blockIdx.x; t < ntiles && !vload(&s_fail); t += gridDim.x) {
-                const TcTile T = tcp_tile(A, t);
-                if (!T.alive) continue;
-                const TcInst& I = A.inst[T.inst];
-                const bool two = I.two_terms != 0;
-                const uint32_t a_bytes = 128u * 128u, b_bytes = (uint32_t)I.bn * 128u;
-                const uint32_t sb = a_bytes + b_bytes * (two ? 2u : 1u);
-                for (int kb = 0; kb < T.kb; ++kb, ++pos, q.next(NS)) {
-                    const int s = q.s;
-                    if (pos >= NS && !mbar_wait(&empty_bar[s], q.par)) {
-                        s_fail = 1;
-                        break;
-                    }
-                    unsigned char* st = ring + (size_t)s * stage_max;
-                    mbar_expect_tx(&full_bar[s], sb);
-                    tma_load_2d(st, &I.tmA, &full_bar[s], 0, (T.mt * T.kb + kb) * 128);
-                    tma_load_2d(st + a_bytes, &I.tmBhi, &full_bar[s], kb * 64, T.nt * I.bn);
-                    if (two) tma_load_2d(st + a_bytes + b_bytes, &I.tmBlo, &full_bar[s], kb * 64, T.nt * I.bn);
-                    s_issued = pos + 1;
+    if (warp == 0 || warp == 8) {
+        // ---- producers: warp 0 of Q_off, warp 8 of the inputs
+        const bool one = elect_one(), of_q = warp == 0;
+        long long pos = 0;
+        RingPos q{0, 1u};   // the first round finds every slot empty
+        for (int t = blockIdx.x; t < ntiles && !uniform((uint32_t)vload(&s_fail)); t += gridDim.x) {
+            const TcTile T = tcp_tile(A, t);
+            if (!T.alive) continue;
+            const TcInst& I = A.inst[T.inst];
+            const bool two = I.two_terms != 0;
+            const uint32_t a_bytes = 128u * 128u, b_bytes = (uint32_t)I.bn * 128u, terms = two ? 2u : 1u;
+            for (int kb = 0; kb < T.kb; kb += KB, ++pos, q.next(NS)) {
+                const int s = q.s;
+                if (pos >= NS && !mbar_wait_warp(&empty_bar[s], q.par)) {
+                    s_fail = 1;
+                    break;
                 }
+                if (one) {
+                    unsigned char* st = ring + (size_t)s * stage_max;
+                    if (of_q) {
+                        mbar_expect_tx(&full_bar[s], (uint32_t)KB * a_bytes);
+                        tma_load_2d(st, KB == 2 ? &I.tmA2 : &I.tmA, &full_bar[s], 0, (T.mt * T.kb + kb) * 128);
+                    } else {
+                        mbar_expect_tx(&full_bar[s], (uint32_t)KB * terms * b_bytes);
+                        for (int k = 0; k < KB; ++k) {
+                            unsigned char* sb = st + (size_t)KB * a_bytes + (size_t)k * terms * b_bytes;
+                            tma_load_2d(sb, &I.tmBhi, &full_bar[s], (kb + k) * 64, T.nt * I.bn);
+                            if (two) tma_load_2d(sb + b_bytes, &I.tmBlo, &full_bar[s], (kb + k) * 64, T.nt * I.bn);
+                        }
+                    }
+                }
+                __syncwarp();
+                s_issued[of_q ? 0 : 1] = pos + 1;
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {   // ---- MMA issuer
-            long long pos = 0;
-            RingPos q{0, 0u};
-            int j = 0;
-            for (int t = blockIdx.x; t < ntiles && !vload(&s_fail); t += gridDim.x) {
-                const TcTile T = tcp_tile(A, t);
-                if (!T.alive) continue;
-                const TcInst& I = A.inst[T.inst];
-                const bool two = I.two_terms != 0;
-                const uint32_t a_bytes = 128u * 128u;
-                const int buf = j & 1, use_b = j >> 1;
-                if (use_b > 0 && !mbar_wait(&acce_bar[buf], (uint32_t)((use_b - 1) & 1))) {
-                    s_fail = 1;
+        // ---- MMA issuer
+        const bool one = elect_one();
+        long long pos = 0;
+        RingPos q{0, 0u};
+        int j = 0;
+        for (int t = blockIdx.x; t < ntiles && !uniform((uint32_t)vload(&s_fail)); t += gridDim.x) {
+            const TcTile T = tcp_tile(A, t);
+            if (!T.alive) continue;
+            const TcInst& I = A.inst[T.inst];
+            const bool two = I.two_terms != 0;
+            const uint32_t a_bytes = 128u * 128u;
+            const int buf = j & 1, use_b = j >> 1;
+            if (use_b > 0 && !mbar_wait_warp(&acce_bar[buf], (uint32_t)((use_b - 1) & 1))) {
+                s_fail = 1;
+                break;
+            }
+            tc_fence_after();
+            const uint32_t d = tmem + (uint32_t)buf * col_stride;
+            const uint32_t idesc = idesc_bf16(128, two ? 2 * I.bn : I.bn);
+            const int NK = tc_chains_k(I.bn);
+            const uint32_t W = (uint32_t)(two ? 2 * I.bn : I.bn);
+            bool ok = true;
+            const uint32_t b_bytes = W * 128u;   // both terms of a k-block
+            for (int kb = 0; kb < T.kb; kb += KB, ++pos, q.next(NS)) {
+                const int s = q.s;
+                if (!mbar_wait_warp(&full_bar[s], q.par)) {
+                    ok = false;
                     break;
                 }
                 tc_fence_after();
-                const uint32_t d = tmem + (uint32_t)buf * col_stride;
-                const uint32_t idesc = idesc_bf16(128, two ? 2 * I.bn : I.bn);
-                const int NK = tc_chains_k(I.bn);
-                const uint32_t W = (uint32_t)(two ? 2 * I.bn : I.bn);
-                bool ok = true;
-                for (int kb = 0; kb < T.kb; ++kb, ++pos, q.next(NS)) {
-                    const int s = q.s;
-                    if (!mbar_wait(&full_bar[s], q.par)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint32_t sa = smem_u32(ring + (size_t)s * stage_max);
-                    umma_kblock(d, sa, sa + a_bytes, idesc, NK, W, kb == 0);
+                const uint32_t sa = uniform(smem_u32(ring + (size_t)s * stage_max));
+                if (one) {
+                    umma_kblock(d, sa, sa + KB * a_bytes, idesc, NK, W, kb == 0);
+                    if (KB == 2) umma_kblock(d, sa + a_bytes, sa + 2 * a_bytes + b_bytes, idesc, NK, W, false);
                     umma_commit(&empty_bar[s]);
                 }
-                if (!ok) {
-                    s_fail = 1;
-                    break;
-                }
-                umma_commit(&accf_bar[buf]);
-                ++j;
+                __syncwarp();
             }
-            // every MMA issued has completed before TMEM is released
-            if (pos > 0) {
-                umma_commit(&fin_bar);
-                mbar_wait(&fin_bar, 0u);
+            if (!ok) {
+                s_fail = 1;
+                break;
             }
+            if (one) umma_commit(&accf_bar[buf]);
+            ++j;
+        }
+        // every MMA issued has completed before TMEM is released
+        if (pos > 0) {
+            if (one) umma_commit(&fin_bar);
+            mbar_wait(&fin_bar, 0u);
         }
     } else {
         // ---- warps 2..7: epilogue; warps 4..7 first drain TMEM into P[col][row]
@@ -928,7 +982,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) phase_a_tcp_kernel(TcArgs A, in
     if (threadIdx.x == 0 && s_fail) {
         if (A.err) atomicExch(A.err, 1);
         // copies already issued land before the ring's shared memory goes away
-        const long long iss = s_issued;
+        const long long iss = s_issued[0] > s_issued[1] ? s_issued[0] : s_issued[1];
         for (long long q = (iss > NS ? iss - NS : 0); q < iss; ++q)
             mbar_wait(&full_bar[q % NS], (uint32_t)((q / NS) & 1));
     }
@@ -964,21 +1018,26 @@ int tc_pick_stages(int bn, bool two)
     return s;
 }
 
-// persistent kernel: ring of `stages` slots of the largest stage, then P (max_bn x 128 FP32)
-size_t tcp_smem_bytes(int bn, bool two, int stages)
+// persistent kernel: ring of `stages` slots of kbs k-blocks of the widest tile, then P (max_bn x 128
+// FP32)
+size_t tcp_smem_bytes(int bn, bool two, int kbs, int stages)
 {
-    const size_t stage = 128 * 128 + (size_t)bn * 128 * (two ? 2 : 1);
+    const size_t stage = kbs * (128 * 128 + (size_t)bn * 128 * (two ? 2 : 1));
     return stage * stages + (size_t)bn * 128 * 4 + 1024;
 }
 
-int tcp_pick_stages(int bn, bool two)
+static int tcp_slots(int bn, bool two, int kbs)
 {
-    const size_t stage = 128 * 128 + (size_t)bn * 128 * (two ? 2 : 1);
+    const size_t stage = kbs * (128 * 128 + (size_t)bn * 128 * (two ? 2 : 1));
     const size_t room = 210 * 1024 - (size_t)bn * 128 * 4 - 1024;
-    int s = (int)(room / stage);
-    if (s > kTcpMaxStages) s = kTcpMaxStages;
-    return s;   // < 2: the persistent kernel does not fit this tile width
+    return std::min((int)(room / stage), kTcpMaxStages);
 }
+
+// two k-blocks per slot where at least three such slots fit (copies in flight while one is used)
+int tcp_pick_kbs(int bn, bool two) { return tcp_slots(bn, two, 2) >= 3 ? 2 : 1; }
+
+// < 2: the persistent kernel does not fit this tile width
+int tcp_pick_stages(int bn, bool two) { return tcp_slots(bn, two, tcp_pick_kbs(bn, two)); }
 
 // two accumulator buffers of terms x chains x bn <= 128 per term columns each
 int tcp_tmem_cols(bool two) { return two ? 512 : 256; }
@@ -986,12 +1045,12 @@ int tcp_tmem_cols(bool two) { return two ? 512 : 256; }
 // one CTA per SM (as many as fit), never more than the tiles
 int tcp_grid(const TcArgs& a, int ntiles)
 {
-    const size_t smem = tcp_smem_bytes(a.max_bn, a.two_any != 0, a.stages);
+    const size_t smem = tcp_smem_bytes(a.max_bn, a.two_any != 0, a.kbs, a.stages);
     int dev = 0, sms = 148, per = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (cudaFuncSetAttribute(phase_a_tcp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, phase_a_tcp_kernel, kTcThreads, smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, phase_a_tcp_kernel, kTcpThreads, smem) != cudaSuccess ||
         per < 1) {
         cudaGetLastError();
         per = 1;
@@ -1002,10 +1061,10 @@ int tcp_grid(const TcArgs& a, int ntiles)
 
 cudaError_t tcp_launch(const TcArgs& a, int ntiles, int grid, cudaStream_t st)
 {
-    const size_t smem = tcp_smem_bytes(a.max_bn, a.two_any != 0, a.stages);
+    const size_t smem = tcp_smem_bytes(a.max_bn, a.two_any != 0, a.kbs, a.stages);
     cudaError_t e = cudaFuncSetAttribute(phase_a_tcp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    phase_a_tcp_kernel<<<grid, kTcThreads, smem, st>>>(a, ntiles);
+    phase_a_tcp_kernel<<<grid, kTcpThreads, smem, st>>>(a, ntiles);
     return cudaGetLastError();
 }
 
@@ -1142,6 +1201,7 @@ extern "C" int ubqp_tc_matmul_probe(const uint16_t* A, const uint16_t* Bhi, cons
         TcInst h;
         memset(&h, 0, sizeof(h));
         if (tc_encode_map(&h.tmA, buf, (int64_t)ld * ld / 64, 64, 128) != CUDA_SUCCESS ||
+            tc_encode_map(&h.tmA2, buf, (int64_t)ld * ld / 64, 64, 256) != CUDA_SUCCESS ||
             tc_encode_map(&h.tmBhi, buf + off_bhi, rows_b, ld, bn) != CUDA_SUCCESS ||
             tc_encode_map(&h.tmBlo, buf + off_blo, rows_b, ld, bn) != CUDA_SUCCESS) {
             rc = UBQP_ECUDA;
@@ -1164,6 +1224,7 @@ extern "C" int ubqp_tc_matmul_probe(const uint16_t* A, const uint16_t* Bhi, cons
         const bool persistent = cluster == -1;
         if (persistent && tcp_pick_stages(bn, two) < 2) { rc = UBQP_ENOTSUP; break; }
         a.stages = persistent ? tcp_pick_stages(bn, two) : tc_pick_stages(bn, two);
+        a.kbs = persistent ? tcp_pick_kbs(bn, two) : 1;
         a.tmem_cols = persistent ? tcp_tmem_cols(two) : tc_tmem_cols(bn, two);
         a.max_bn = bn;
         a.two_any = two ? 1 : 0;

@@ -17,6 +17,7 @@ constexpr int kTcMaxCluster = 8;   // CTAs per split-K cluster
 struct alignas(128) TcInst {
     CUtensorMap tmA;     // Q_off in the tiled layout (qbf_index): a (ld*ld/64) x 64 view,
                          // box 64 x 128 = one contiguous 16 KB tile
+    CUtensorMap tmA2;    // the same with two k-blocks of an M tile per box (32 KB)
     CUtensorMap tmBhi;   // lane inputs (hi term), box 64 x bn
     CUtensorMap tmBlo;   // lane inputs (lo term), box 64 x bn
     int32_t n, ld, R, lane0;
@@ -29,7 +30,8 @@ struct alignas(128) TcInst {
 struct TcArgs {
     const TcInst* inst;
     int32_t ninst;
-    int32_t stages;
+    int32_t stages;      // ring slots
+    int32_t kbs;         // k-blocks per ring slot (persistent kernel: 1 or 2)
     int32_t tmem_cols;
     int32_t max_bn;
     int32_t two_any;     // some instance carries the lo term (shared-memory sizing)
@@ -51,8 +53,9 @@ int tc_tmem_cols(int bn, bool two);
 CUresult tc_encode_map(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, int box_rows);
 
 // persistent kernel (many tiles, no split-K)
-size_t tcp_smem_bytes(int bn, bool two, int stages);
-int tcp_pick_stages(int bn, bool two);
+size_t tcp_smem_bytes(int bn, bool two, int kbs, int stages);
+int tcp_pick_kbs(int bn, bool two);
+int tcp_pick_stages(int bn, bool two);   // slots of tcp_pick_kbs k-blocks
 int tcp_tmem_cols(bool two);
 int tcp_grid(const TcArgs& a, int ntiles);
 cudaError_t tcp_launch(const TcArgs& a, int ntiles, int grid, cudaStream_t st);
