@@ -123,6 +123,74 @@ __device__ __forceinline__ double row_dot_eval(const float2* __restrict__ row, c
     return ((double)ah.x + (double)ah.y) + ((double)al.x + (double)al.y);
 }
 
+// NR rows of the evaluation matrix (row stride ld, the first `valid` exist) at once, 4 NR 16-byte
+// loads in flight per lane; every row's entries in row_dot_eval's order.  For kernels with the
+// registers: a row at a time is a chain of trips to memory (a block of 32 rows of n = 2500 took 43,000
+// cycles of an eight-warp CTA)
+template <int NR>
+__device__ __forceinline__ void rows_dot_eval(const float2* __restrict__ rows, int ld, int valid, const float* su, int lane,
+                                              double (&out)[NR], int stride)
+{
+    const float2* u2 = reinterpret_cast<const float2*>(su);
+    const int n2 = ld >> 1;
+    const float4* r4[NR];
+    float2 ah[NR], al[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        r4[r] = reinterpret_cast<const float4*>(rows + (size_t)(r < valid ? r * stride : 0) * ld);
+        ah[r] = al[r] = make_float2(0.f, 0.f);
+    }
+    int c = lane;
+    for (; c + 96 < n2; c += 128) {
+        float4 q[NR][4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int r = 0; r < NR; ++r) q[r][j] = ldg_stream(r4[r] + c + 32 * j);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float2 u = u2[c + 32 * j];
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+                if (u.x != 0.f) { csum_add(ah[r], q[r][j].x); csum_add(al[r], q[r][j].y); }
+                if (u.y != 0.f) { csum_add(ah[r], q[r][j].z); csum_add(al[r], q[r][j].w); }
+            }
+        }
+    }
+    for (; c < n2; c += 32) {
+        const float2 u = u2[c];
+        float4 q[NR];
+#pragma unroll
+        for (int r = 0; r < NR; ++r) q[r] = ldg_stream(r4[r] + c);
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            if (u.x != 0.f) { csum_add(ah[r], q[r].x); csum_add(al[r], q[r].y); }
+            if (u.y != 0.f) { csum_add(ah[r], q[r].z); csum_add(al[r], q[r].w); }
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        ah[r] = csum_shfl_reduce(ah[r]);
+        al[r] = csum_shfl_reduce(al[r]);
+        out[r] = ((double)ah[r].x + (double)ah[r].y) + ((double)al[r].x + (double)al[r].y);
+    }
+}
+
+// the rows row0 .. row0 + rows of the evaluation matrix, four at a time per warp, into sv
+__device__ __forceinline__ void item_rows_eval(const LaneDev& L, int row0, int rows, const float* su, double* sv, int lane,
+                                               int warp)
+{
+    for (int r = warp; r < rows; r += 4 * kWarps) {
+        double v[4];
+        const int valid = (rows - r + kWarps - 1) / kWarps;   // of the rows r, r + 8, r + 16, r + 24
+        rows_dot_eval<4>(L.Qeval + (size_t)(row0 + r) * L.ld, L.ld, valid, su, lane, v, kWarps);
+        if (lane == 0)
+#pragma unroll
+            for (int h = 0; h < 4; ++h)
+                if (h < valid) sv[r + h * kWarps] = v[h];
+    }
+}
+
 // u (written by the lane's last update, zero beyond n) into shared memory
 __device__ __forceinline__ void item_load_u(const LaneDev& L, float* su)
 {

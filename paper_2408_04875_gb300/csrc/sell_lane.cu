@@ -686,13 +686,26 @@ __global__ void __launch_bounds__(kThreads, kPer) sell_lane_kernel(SoloArgs A)
                 // ================= every other step: the shared functions between group barriers
                 item_load_u(L, su);
                 __syncthreads();
-                for (int blk = rank; blk < nblk; blk += nc) {
-                    const int row0 = blk * A.rows_per_item;
-                    const int rows = min(A.rows_per_item, n - row0);
-                    item_rows_solver(L, ph, row0, rows, su, sv, lane, warp);
+                if (ph == PH_EVAL) {
+                    for (int blk = rank; blk < nblk; blk += nc) {
+                        const int row0 = blk * A.rows_per_item;
+                        const int rows = min(A.rows_per_item, n - row0);
+                        item_rows_eval(L, row0, rows, su, sv, lane, warp);
+                        __syncthreads();
+                        item_finish(L, ph, S.k, blk, row0, rows, sv, P);
+                        __syncthreads();
+                    }
+                } else {
+                    // the products of all slices first, then the blocks' epilogues
+                    products();
                     __syncthreads();
-                    item_finish(L, ph, S.k, blk, row0, rows, sv, P);
+                    if (own_warp) sv[tid] = (double)own_product();
                     __syncthreads();
+                    for (int b = 0; b < (one ? 1 : sl.n); ++b) {
+                        const int blk = one ? 0 : sl.at(b), row0 = 32 * blk;
+                        item_finish(L, ph, S.k, blk, row0, one ? n : min(32, n - row0), sv + 32 * b, P);
+                        __syncthreads();
+                    }
                 }
                 if (!solo_grid_sync(A, bar, nc, gen, &s_ok)) break;
                 reduce_partials(L.part, nblk, ph, R);

@@ -596,7 +596,7 @@ __global__ void __launch_bounds__(kThreads, 1) sym_lane_kernel(SoloArgs A)
                 item_load_u(L, su);
                 __syncthreads();
                 if (ph == PH_EVAL) {
-                    if (has_blk) item_rows_solver(L, ph, rank * kBlkRows, rows, su, sv, lane, warp);
+                    if (has_blk) item_rows_eval(L, rank * kBlkRows, rows, su, sv, lane, warp);
                 } else {
                     const float v = product((uint32_t)S.updates);
                     if (tid < rows) sv[tid] = (double)v;
