@@ -35,13 +35,20 @@ namespace ubqp {
 namespace {
 
 constexpr int kTcpThreads = 288;      // persistent kernel: a ninth warp copies the inputs
-constexpr int kTcThreads = 256;       // 8 warps: TMA producer, MMA issuer, then all 8 drain TMEM / run the epilogue
+// split-K kernel: TMA producer, MMA issuer, then all warps drain TMEM and run the epilogue.  16 warps up
+// to four CTAs per cluster; with more, a thread's prefetched partials need the registers of 8.
+constexpr int kTcThreads = 512;
+constexpr int kTcThreadsWide = 256;
+constexpr int kTcWideFrom = 5;        // cluster size from which the 8-warp form runs
 constexpr uint64_t kWaitNs = 2000000000ull;
-// split-K kernel epilogue: each warp stages the operand rows of its next kEpiDepth lanes in
-// shared memory (slots of kEpiSlot floats = 7 vectors x 128 rows, after the accumulators)
-constexpr int kEpiDepth = 3;
+// split-K kernel epilogue: each warp stages the operand rows of its next kEpiDepth (8-warp form:
+// kEpiDepthWide) lanes in shared memory (slots of kEpiSlot floats = 7 vectors x 128 rows, after
+// the accumulators)
+constexpr int kEpiDepth = 2;
+constexpr int kEpiDepthWide = 3;
 constexpr int kEpiSlot = 7 * 128;
 constexpr size_t kEpiSlotBytes = (size_t)(kTcThreads / 32) * kEpiDepth * kEpiSlot * 4;
+static_assert(kTcThreadsWide * kEpiDepthWide <= kTcThreads * kEpiDepth, "the slots of either form fit");
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -454,7 +461,9 @@ __device__ __forceinline__ void tc_fused_count(const TcArgs& A, const LaneDev& L
 }
 
 // ---------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kTcThreads, 1) phase_a_tc_kernel(TcArgs A)
+// kS: largest cluster size this instance serves (registers for the partials of kS ranks)
+template <int kS, int kThr, int kDepth>
+__global__ void __launch_bounds__(kThr, 1) phase_a_tc_kernel(TcArgs A)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // 1024-byte aligned ring
@@ -463,7 +472,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) phase_a_tc_kernel(TcArgs A)
     __shared__ uint32_t tmem_base;
     __shared__ int s_inst, s_mt, s_nt, s_skip;
     __shared__ int s_fail;
-    __shared__ WarpUpd s_upd[kTcThreads / 32];
+    __shared__ WarpUpd s_upd[kThr / 32];
 
     cg::cluster_group cluster = cg::this_cluster();
     const int S = (int)cluster.num_blocks();
@@ -530,7 +539,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) phase_a_tc_kernel(TcArgs A)
     const int nreal = min(BN, I.R - nt * BN);
     const int c0 = (int)((int64_t)nreal * rank / S), c1 = (int)((int64_t)nreal * (rank + 1) / S);
     if (!s_skip && !A.raw && warp >= 2)
-        for (int c = c0 + (int)threadIdx.x - 64; c < c1; c += kTcThreads - 64) {
+        for (int c = c0 + (int)threadIdx.x - 64; c < c1; c += kThr - 64) {
             const LaneDev& Ld = A.lanes[I.lane0 + nt * BN + c];
             const LaneState* st = Ld.st;
             s_ph[c - c0] = st->phase;
@@ -595,12 +604,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) phase_a_tc_kernel(TcArgs A)
     __syncthreads();
     float* P = reinterpret_cast<float*>(ring);
     // operand slots after the accumulators (the ring is free now); warp w's lanes are
-    // c0 + w + 8 t, lane t in slot t mod kEpiDepth, one copy group per lane
-    float* slots = P + 128 * A.max_bn + (size_t)warp * kEpiDepth * kEpiSlot;
+    // c0 + w + warps * t, lane t in slot t mod kDepth, one copy group per lane
+    float* slots = P + 128 * A.max_bn + (size_t)warp * kDepth * kEpiSlot;
     auto epi_issue = [&](int t) {
-        const int c = c0 + warp + (kTcThreads / 32) * t;
+        const int c = c0 + warp + (kThr / 32) * t;
         if (!A.raw && c < c1 && epi_ops_phase(s_ph[c - c0]))
-            tc_epi_copy(s_epi[c - c0].vec, s_ph[c - c0], I.ld, mt * 128, slots + (t % kEpiDepth) * kEpiSlot, lane);
+            tc_epi_copy(s_epi[c - c0].vec, s_ph[c - c0], I.ld, mt * 128, slots + (t % kDepth) * kEpiSlot, lane);
         cp_async_commit();
     };
     if (!s_skip) {
@@ -613,13 +622,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) phase_a_tc_kernel(TcArgs A)
             cp_async_commit();
         }
 #pragma unroll
-        for (int t = 0; t < kEpiDepth; ++t) epi_issue(t);
+        for (int t = 0; t < kDepth; ++t) epi_issue(t);
     }
     if (!s_skip) {
         const bool have = nkb > 0 && s_ok;
         if (nkb > 0) tc_fence_after();
         const int row = (warp & 3) * 32 + lane;   // TMEM lanes reachable by this warp
-        for (int q = warp >> 2; q < BN / 16; q += 2) {   // 16-column chunks split over the two warpgroups
+        for (int q = warp >> 2; q < BN / 16; q += kThr / 128) {   // 16-column chunks split over the warpgroups
             float v[16];
             if (have) {
                 tmem_ld16_sum(tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(q * 16), BN, two, v);
@@ -651,40 +660,41 @@ __global__ void __launch_bounds__(kTcThreads, 1) phase_a_tc_kernel(TcArgs A)
             if (mt == 0) by += 2ull * (two ? 2ull : 1ull) * (unsigned long long)nreal * (unsigned long long)I.n;
             atomicAdd(A.P.bytes, by);
         }
-        if (!A.raw && threadIdx.x < 64) cp_async_wait<kEpiDepth>();   // the tile's tsum and row sums
+        if (!A.raw && threadIdx.x < 64) cp_async_wait<kDepth>();   // the tile's tsum and row sums
         __syncthreads();
-        float* peers[kTcMaxCluster];
-        for (int q = 0; q < S; ++q) peers[q] = cluster.map_shared_rank(P, q);
-        // lanes c0 + warp, + 8, ...: the operands come from the warp's slots; the next lane's
+        float* peers[kS];
+#pragma unroll
+        for (int q = 0; q < kS; ++q) peers[q] = cluster.map_shared_rank(P, q < S ? q : 0);
+        // lanes c0 + warp, + the warps, ...: the operands come from the warp's slots; the next lane's
         // cluster partials (every rank's value of its four rows, summed in rank order when its
         // turn comes) load while this one finishes
-        float pcur[kTcMaxCluster][4], pnxt[kTcMaxCluster][4];
-        auto load_parts = [&](int c, float (&pv)[kTcMaxCluster][4]) {
+        float pcur[kS][4], pnxt[kS][4];
+        auto load_parts = [&](int c, float (&pv)[kS][4]) {
 #pragma unroll
-            for (int q = 0; q < kTcMaxCluster; ++q)
+            for (int q = 0; q < kS; ++q)
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
                     if (q < S) pv[q][j] = peers[q][c * 128 + lane + 32 * j];
         };
         if (c0 + warp < c1) load_parts(c0 + warp, pcur);
-        for (int c = c0 + warp, t = 0; c < c1; c += kTcThreads / 32, ++t) {
+        for (int c = c0 + warp, t = 0; c < c1; c += kThr / 32, ++t) {
             const int r = nt * BN + c;  // restart index within the instance
-            const int cn = c + kTcThreads / 32;
+            const int cn = c + kThr / 32;
             if (cn < c1) load_parts(cn, pnxt);
             const int ph = A.raw ? PH_DONE : s_ph[c - c0];
             const bool staged = epi_ops_phase(ph);
             EpiOps cur;
-            cp_async_wait<kEpiDepth - 1>();   // lane t's group
+            cp_async_wait<kDepth - 1>();   // lane t's group
             __syncwarp();
-            if (staged) tc_epi_from_slot(slots + (t % kEpiDepth) * kEpiSlot, s_rows, ph, lane, cur);
-            __syncwarp();                     // the slot is read: it takes lane t + kEpiDepth
-            epi_issue(t + kEpiDepth);
+            if (staged) tc_epi_from_slot(slots + (t % kDepth) * kEpiSlot, s_rows, ph, lane, cur);
+            __syncwarp();                     // the slot is read: it takes lane t + kDepth
+            epi_issue(t + kDepth);
             float vv[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 float acc = 0.f;
 #pragma unroll
-                for (int q = 0; q < kTcMaxCluster; ++q)
+                for (int q = 0; q < kS; ++q)
                     if (q < S) acc += pcur[q][j];
                 vv[j] = acc;
             }
@@ -700,7 +710,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) phase_a_tc_kernel(TcArgs A)
                 if (A.fuse) tc_fused_count(A, A.lanes[I.lane0 + r], s_upd[warp]);
             }
 #pragma unroll
-            for (int q = 0; q < kTcMaxCluster; ++q)
+            for (int q = 0; q < kS; ++q)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) pcur[q][j] = pnxt[q][j];
         }
@@ -782,7 +792,7 @@ __global__ void __launch_bounds__(kTcpThreads, 1) phase_a_tcp_kernel(TcArgs A, i
     __shared__ uint32_t tmem_base;
     __shared__ int s_fail;
     __shared__ long long s_issued[2];
-    __shared__ WarpUpd s_upd[kTcThreads / 32];
+    __shared__ WarpUpd s_upd[kTcpThreads / 32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t col_stride = A.two_any ? 256u : 128u;   // one accumulator buffer: terms x chains x bn <= this
 
@@ -1068,44 +1078,49 @@ cudaError_t tcp_launch(const TcArgs& a, int ntiles, int grid, cudaStream_t st)
     return cudaGetLastError();
 }
 
-cudaError_t tc_launch(const TcArgs& a, int total_clusters, int S, cudaStream_t st)
+typedef void (*TcKernel)(TcArgs);
+static TcKernel tc_kernel(int S)
 {
-    size_t smem = tc_smem_bytes(a.max_bn, a.two_any != 0, a.stages);
-    cudaError_t e = cudaFuncSetAttribute(phase_a_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    if (S >= kTcWideFrom) return phase_a_tc_kernel<kTcMaxCluster, kTcThreadsWide, kEpiDepthWide>;
+    return S <= 2 ? phase_a_tc_kernel<2, kTcThreads, kEpiDepth> : phase_a_tc_kernel<4, kTcThreads, kEpiDepth>;
+}
+
+static cudaLaunchConfig_t tc_config(int ctas, int S, size_t smem, cudaLaunchAttribute* attr)
+{
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(total_clusters * S), 1, 1);
-    cfg.blockDim = dim3(kTcThreads, 1, 1);
+    cfg.gridDim = dim3((unsigned)ctas, 1, 1);
+    cfg.blockDim = dim3(S >= kTcWideFrom ? kTcThreadsWide : kTcThreads);
     cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)S;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = (unsigned)S;
+    attr->val.clusterDim.y = 1;
+    attr->val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, phase_a_tc_kernel, a);
+    return cfg;
+}
+
+cudaError_t tc_launch(const TcArgs& a, int total_clusters, int S, cudaStream_t st)
+{
+    const size_t smem = tc_smem_bytes(a.max_bn, a.two_any != 0, a.stages);
+    const TcKernel k = tc_kernel(S);
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg = tc_config(total_clusters * S, S, smem, attr);
+    cfg.stream = st;
+    return cudaLaunchKernelEx(&cfg, k, a);
 }
 
 int tc_max_active_clusters(int bn, bool two, int stages, int S)
 {
-    size_t smem = tc_smem_bytes(bn, two, stages);
-    if (cudaFuncSetAttribute(phase_a_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return 0;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(S * 64), 1, 1);
-    cfg.blockDim = dim3(kTcThreads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
+    const size_t smem = tc_smem_bytes(bn, two, stages);
+    const TcKernel k = tc_kernel(S);
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)S;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    const cudaLaunchConfig_t cfg = tc_config(S * 64, S, smem, attr);
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, phase_a_tc_kernel, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
