@@ -249,6 +249,67 @@ __device__ __forceinline__ void tmem_ld16_sum(uint32_t taddr, int bn, bool two, 
         }
 }
 
+// Butterfly of N compensated sums that halves what a thread holds at every level: at distance o the
+// threads with bit o set keep the second half of their sums and hand over the first, the others
+// the reverse.  Every sum meets the same pairs of partial sums as in the plain butterfly (and TwoSum
+// does not mind which of a pair is its first operand), so it has the same bits, from 13 merges
+// instead of 60 for twelve sums.  Returns this thread's sum, number `idx` (>= N: none); threads
+// that differ only in the bits of levels with a single sum hold the same one.
+template <int N, int O>
+__device__ __forceinline__ float2 halving_sum(const float2 (&s)[N], int& idx)
+{
+    if constexpr (O == 0) {
+        return s[0];
+    } else if constexpr (N == 1) {
+        float2 w;
+        w.x = __shfl_xor_sync(0xffffffffu, s[0].x, O);
+        w.y = __shfl_xor_sync(0xffffffffu, s[0].y, O);
+        const float2 m[1] = {csum_merge(s[0], w)};
+        return halving_sum<1, O / 2>(m, idx);
+    } else {
+        constexpr int H = (N + 1) / 2;
+        const bool up = threadIdx.x & O;
+        float2 m[H];
+#pragma unroll
+        for (int t = 0; t < H; ++t) {
+            const float2 a = s[t], b = t + H < N ? s[t + H < N ? t + H : 0] : make_float2(0.f, 0.f);
+            float2 w;
+            w.x = __shfl_xor_sync(0xffffffffu, up ? a.x : b.x, O);
+            w.y = __shfl_xor_sync(0xffffffffu, up ? a.y : b.y, O);
+            m[t] = csum_merge(up ? b : a, w);
+        }
+        int sub = 0;
+        const float2 r = halving_sum<H, O / 2>(m, sub);
+        idx = up ? (sub < N - H ? H + sub : N) : (sub < H ? sub : N);
+        return r;
+    }
+}
+
+// the records of the two steps that repeat: the gradient step's three sums and maxima (the first step
+// of a subproblem, k = 0, has maxima only in 1 .. 3, the others only in 0) and the eigen-solver's
+// twelve sums.  Records hold what their phase's reduction reads.
+__device__ __forceinline__ void warp_write_inner(const float2 (&s)[3], float (&m)[4], int k, Partial* out)
+{
+    int idx = 0;
+    const float2 v = halving_sum<3, 16>(s, idx);
+    if (idx < 3 && (threadIdx.x & 7) == 0) out->s[idx] = v;
+    if (k >= 1) {
+        m[0] = max_shfl_reduce(m[0]);
+    } else {
+#pragma unroll
+        for (int t = 0; t < 4; ++t) m[t] = max_shfl_reduce(m[t]);
+    }
+    if ((threadIdx.x & 31) == 0)
+#pragma unroll
+        for (int t = 0; t < 4; ++t) out->m[t] = m[t];
+}
+__device__ __forceinline__ void warp_write_gram(const float2 (&s)[12], Partial* out)
+{
+    int idx = 0;
+    const float2 v = halving_sum<12, 16>(s, idx);
+    if (idx < 12 && (threadIdx.x & 1) == 0) out->s[idx] = v;
+}
+
 // warp-level reduction of one lane's accumulator into its partial record (lane 0 writes)
 __device__ __forceinline__ void warp_reduce_write(Acc& a, int ph, Partial* out, bool has_f)
 {
@@ -333,7 +394,9 @@ __device__ __forceinline__ void tc_epi_finish(float* vec, Partial* part, int ph,
             const float viol = (x > 0.f && x < 1.f) ? fabsf(g) : (x <= 0.f ? fmaxf(-g, 0.f) : fmaxf(g, 0.f));
             a.m[0] = fmaxf(a.m[0], viol);
         }
-        warp_reduce_write(a, PH_INNER, part + mt, false);
+        const float2 s3[3] = {a.s[0], a.s[1], a.s[2]};
+        float m4[4] = {a.m[0], a.m[1], a.m[2], a.m[3]};
+        warp_write_inner(s3, m4, k, part + mt);
         return;
     }
 #pragma unroll
@@ -363,7 +426,8 @@ __device__ __forceinline__ void tc_epi_finish(float* vec, Partial* part, int ph,
             csum_add(a.s[11], p * p);
         }
     }
-    warp_reduce_write(a, ph, part + mt, false);
+    if (ph == PH_LOB) warp_write_gram(a.s, part + mt);
+    else warp_reduce_write(a, ph, part + mt, false);
 }
 
 // the fields of a lane's descriptor that the prefetched epilogues use
