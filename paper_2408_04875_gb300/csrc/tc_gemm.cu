@@ -34,7 +34,8 @@ namespace ubqp {
 
 namespace {
 
-constexpr int kTcpThreads = 288;      // persistent kernel: a ninth warp copies the inputs
+constexpr int kTcpThreads = 352;      // persistent kernel: 3 warps feed the tensor core, 8 run the epilogue
+constexpr int kTcpEpiWarps = kTcpThreads / 32 - 3;
 // split-K kernel: TMA producer, MMA issuer, then all warps drain TMEM and run the epilogue.  16 warps up
 // to four CTAs per cluster; with more, a thread's prefetched partials need the registers of 8.
 constexpr int kTcThreads = 512;
@@ -801,7 +802,10 @@ __global__ void __launch_bounds__(kThr, 1) phase_a_tc_kernel(TcArgs A)
 // one k-block per slot its instructions set the pace, 600 cycles a k-block); warp 1 issues the MMAs of each tile into one of two TMEM accumulators (columns
 // buf * max_bn), waiting until the epilogue has drained that buffer; warps 4..7 drain the
 // finished accumulator into shared memory (each warp reaches TMEM lanes 32 (w mod 4) ..)
-// and release it; warps 2..7 then run the per-row epilogue of the tile's lanes.  All roles
+// and release it; warps 2..7, 9 and 10 then run the per-row epilogue of the tile's lanes, eight
+// at a time (registers are given out to four warps at once: the eleven cost
+// what nine would; six epilogue warps took eight starts in two turns: 27.4 us a step of the
+// ragged batch, eight 26.2).  All roles
 // walk the same tile list and skip the same finished tiles (lane states do not change
 // during the launch).  Waits are bounded; after a failure every role stops working but the
 // epilogue warps keep their named barriers matched, and the CTA lets issued copies and
@@ -851,7 +855,7 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar)
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
-__device__ __forceinline__ void epi_bar_sync() { asm volatile("bar.sync 1, 192;" ::: "memory"); }
+__device__ __forceinline__ void epi_bar_sync() { asm volatile("bar.sync 1, %0;" ::"n"(32 * kTcpEpiWarps) : "memory"); }
 
 __device__ __forceinline__ int vload(const int* p) { return *reinterpret_cast<const volatile int*>(p); }
 
@@ -978,8 +982,9 @@ __global__ void __launch_bounds__(kTcpThreads, 1) phase_a_tcp_kernel(TcArgs A, i
             mbar_wait(&fin_bar, 0u);
         }
     } else {
-        // ---- warps 2..7: epilogue; warps 4..7 first drain TMEM into P[col][row]
-        const bool drain = warp >= 4;
+        // ---- warps 2..7, 9, 10: epilogue; warps 4..7 first drain TMEM into P[col][row]
+        const bool drain = warp >= 4 && warp < 8;
+        const int ew = warp < 8 ? warp - 2 : warp - 3;
         int j = 0;
         for (int rd = 0, t; (t = tcp_pick(rd)) < ntiles; ++rd) {
             const TcTile T = tcp_tile(A, t);
@@ -1024,7 +1029,7 @@ __global__ void __launch_bounds__(kTcpThreads, 1) phase_a_tcp_kernel(TcArgs A, i
                         atomicAdd(A.P.bytes, by);
                     }
                 }
-                // lanes warp - 2, + 6, ...: the next lane's operands load while this one finishes
+                // lanes ew, ew + kTcpEpiWarps, ...: the next lane's operands load while this one finishes
                 EpiOps cur, nxt;
                 int cur_ph = PH_DONE, cur_k = 0;
                 auto lane_at = [&](int c, EpiOps& o, int& ph, int& k) {
@@ -1036,11 +1041,11 @@ __global__ void __launch_bounds__(kTcpThreads, 1) phase_a_tcp_kernel(TcArgs A, i
                     k = st->k;
                     if (epi_ops_phase(ph)) tc_epi_load(L.vec, L.tsum, L.oabs, ph, I.ld, I.n, T.mt, lane, o);
                 };
-                lane_at(warp - 2, cur, cur_ph, cur_k);
-                for (int c = warp - 2; c < nreal; c += 6) {
+                lane_at(ew, cur, cur_ph, cur_k);
+                for (int c = ew; c < nreal; c += kTcpEpiWarps) {
                     const int r = T.nt * I.bn + c;
                     int nxt_ph, nxt_k = 0;
-                    lane_at(c + 6, nxt, nxt_ph, nxt_k);
+                    lane_at(c + kTcpEpiWarps, nxt, nxt_ph, nxt_k);
                     float vv[4];
 #pragma unroll
                     for (int q = 0; q < 4; ++q) vv[q] = P[c * 128 + lane + 32 * q];
