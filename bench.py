@@ -30,12 +30,13 @@ sys.path.insert(0, ROOT)
 
 METRIC = "inner PG iters/s (batch×n) and time-to-oracle-objective vs plain FP32 path"
 UNIT = "lane-var-updates/s"
-GEMV_KERNELS = {1: "phase_a_gemv_kernel", 2: "lane_loop_kernel", 3: "solo_lane_kernel"}
+GEMV_KERNELS = {1: "phase_a_gemv_kernel", 2: "lane_loop_kernel", 3: "sell_lane_kernel"}
 # DRAM bytes (read + write) per algorithmic byte of the dominant kernel, keyed by (scheduler,
 # storage), from an ncu capture of every launch of this workload's timed solve
 # (dram__bytes_read.sum + dram__bytes_write.sum over the launches against the bench's own
-# algorithmic bytes; the C2 launch list under profiles/); other combinations report null
-TRAFFIC_RATIO = {(3, 2): 0.7935 / 37.774}
+# algorithmic bytes); combinations without such a capture report null (the lane-group kernels have
+# one of a capped sweep only, under profiles/)
+TRAFFIC_RATIO = {}
 SIZES = (250, 500, 1000, 2500)
 SEEDS_PER_SIZE = 10
 WORKLOAD = ("plain PSDP sweep: n in {250,500,1000,2500} x 10 seeded instances, density 0.1, "
@@ -241,9 +242,9 @@ C3_WORKLOAD = ("differentiable objective: n=1000 dense Q in [-100,100], b in [-5
 def run_c3(args):
     """The penalized objective and its gradient (the autograd forward) on the 64 C3 points,
     FP32 and FP64: value = gradient entries per second (64 x n per call).  Each call is timed
-    with CUDA events on its stream (the entry point's scratch set-up, the GEMV kernel and the
+    with CUDA events on its stream (the entry point's scratch set-up, the tile kernel and the
     reduction of h).  Algorithmic bytes: Q once per call plus the points and gradients; the
-    kernel reads Q once per point, from L2 after the first (reported as l2_bytes_per_call)."""
+    kernel reads Q once per eight points, from L2 after the first (reported as l2_bytes_per_call)."""
     import numpy as np
     import torch
     import paper_2408_04875_gb300 as ub
@@ -272,7 +273,7 @@ def run_c3(args):
         alg = es * (1000 * 1000 + 3 * 1000 + 2 * 64 * 1000) + es * 64
         out[name] = {"us_per_call": t * 1e6, "value": 64 * 1000 / t, "algorithmic_bytes_per_call": alg,
                      "achieved_gbs": alg / t / 1e9, "frac_hbm": alg / t / 1e9 / peak,
-                     "l2_bytes_per_call": 64 * es * 1000 * 1000, "l2_gbs": 64 * es * 1e6 / t / 1e9,
+                     "l2_bytes_per_call": 8 * es * 1000 * 1000, "l2_gbs": 8 * es * 1e6 / t / 1e9,
                      "fp_gflops": 2 * 64 * 1e6 / t / 1e9}
     line = {"metric": "penalized objective + gradient entries/s", "value": out["f32"]["value"],
             "unit": "gradient entries/s", "n_gpus": 1, "steps": args.steps, "warmup": args.warmup,
@@ -280,7 +281,7 @@ def run_c3(args):
             "vs_baseline": None, "dtype": "f32", "data": "synthetic",
             "config": {"workload": C3_WORKLOAD, "f64": out["f64"], "l2": "Q (4 MB FP32) is L2-resident"},
             "roofline": {"bound": "hbm", "achieved": out["f32"]["achieved_gbs"], "peak": peak, "unit": "GB/s",
-                         "frac": out["f32"]["frac_hbm"], "traffic": None, "kernel": "phase_a_gemv_kernel",
+                         "frac": out["f32"]["frac_hbm"], "traffic": None, "kernel": "grad_kernel",
                          "peak_kind": peak_kind, "f32": out["f32"]}}
     print(json.dumps(line), flush=True)
     return 0
@@ -359,9 +360,9 @@ SINGLE_WORKLOAD = ("plain FP32 path, one lane: C1 (n=50, density 0.1, seed 0) an
 
 
 def run_single(args):
-    """The plain FP32 single-instance path: whole solves of one lane on the single-lane persistent
-    kernel (gemv_kernel = 3) and on the lock-step scheduler (gemv_kernel = 1), device time per
-    step.  Roofline of the single-lane kernel at n = 2500: algorithmic bytes per step (the sparse
+    """The plain FP32 single-instance path: whole solves of one lane on its own group of
+    CTAs (gemv_kernel = 3) and on the lock-step scheduler (gemv_kernel = 1), device time per
+    step.  Roofline of the group kernel at n = 2500: algorithmic bytes per step (the sparse
     minimum, 6 B per stored entry + 32 B per row) over the time per step, against HBM (the
     sliced storage of one lane, 3.8 MB, is L2-resident, so the fraction can exceed 1)."""
     import torch
@@ -393,7 +394,7 @@ def run_single(args):
             "ms_per_step": big["ms"], "higher_is_better": False, "scaling": "weak", "vs_baseline": None,
             "dtype": "f32", "data": "synthetic", "config": {"workload": SINGLE_WORKLOAD, "results": out},
             "roofline": {"bound": "hbm", "achieved": big["achieved_gbs"], "peak": peak, "unit": "GB/s",
-                         "frac": big["achieved_gbs"] / peak, "traffic": None, "kernel": "solo_lane_kernel",
+                         "frac": big["achieved_gbs"] / peak, "traffic": None, "kernel": "sell_lane_kernel",
                          "peak_kind": peak_kind, "l2": "the lane's sliced storage is L2-resident"}}
     print(json.dumps(line), flush=True)
     return 0

@@ -79,7 +79,7 @@ typedef struct {
     int64_t phase_a_flops;   /* algorithmic flops of the tensor-core launches timed     */
     int32_t cluster_size;    /* CTAs per cluster of the tensor-core launches (0: none)  */
     int32_t gemv_kernel;     /* scheduler that ran the FP32 lanes: 1 lock-step, 2 lane  */
-                             /* loop, 3 single-lane kernel (0: tensor-core lanes)       */
+                             /* loop, 3 lane groups (0: tensor-core lanes)              */
     int32_t restarts;        /* starts per instance that ran (the tuner's pick when     */
                              /* opts->restarts == 0)                                    */
     float restart_probe_us[5]; /* restart tuner: step time measured with 1, 8, 32, 64  */
@@ -145,25 +145,27 @@ typedef struct {
                              /* UBQP_TUNE_CACHE names a file, in that JSON file          */
     int gemv_kernel;         /* scheduler of the FP32 lanes: 1 lock-step (one launch   */
                              /* per step of all lanes), 2 persistent lane loop (lanes  */
-                             /* advance independently inside one launch), 3 single-lane */
-                             /* persistent kernel (many steps per cooperative launch;  */
-                             /* each lane on its own group of CTAs with a bounded group */
-                             /* barrier, one per PABB step; with more lanes than       */
+                             /* advance independently inside one launch), 3 lane groups  */
+                             /* (many steps per cooperative launch; each lane on its own */
+                             /* group of CTAs, which exchange a step's results by tagged */
+                             /* words or a bounded group barrier; with more lanes than   */
                              /* resident CTAs, one-CTA groups run several lanes in      */
-                             /* turn); 0 = 3 for one lane and for lanes on the sliced   */
-                             /* storage whose groups fit with at most 5 slices per CTA, */
-                             /* else 2 for 4 or more lanes, else 1 (1 when              */
-                             /* profile_kernels == 2); UBQP_ENOTSUP when 3 is asked for */
-                             /* and a lane's two vectors exceed 200 KiB of shared memory */
-    int lane_budget;         /* lane loop and single-lane kernel: steps per lane (per   */
+                             /* turn); 0 = 3 for one lane, for lanes on the sliced      */
+                             /* storage whose groups fit with at most 5 slices per CTA  */
+                             /* and for 4 or more lanes on the symmetric tiles whose    */
+                             /* groups fit with at most 20 tiles per CTA, else 2 for 4   */
+                             /* or more lanes, else 1 (1 when profile_kernels == 2);     */
+                             /* UBQP_ENOTSUP when 3 is asked for and a lane's two        */
+                             /* vectors exceed 200 KiB of shared memory                  */
+    int lane_budget;         /* lane loop and lane groups: steps per lane (per          */
                              /* group) between host checks; 0 = 1024                    */
     int rows_per_item;       /* FP32 lanes: matrix rows per work item, 8..256 (a multiple */
                              /* of 8); 0 = chosen from the batch size                  */
-    int sym_storage;         /* FP32 lanes on the lane loop: 1 = store only the upper   */
+    int sym_storage;         /* FP32 lanes in groups or on the lane loop: 1 = store only the upper */
                              /* triangle of Q'_off (128 x 128 tiles; each step reads    */
                              /* about half the bytes), 0 = dense rows: 1                */
-    int wait_limit_us;       /* lane loop and single-lane kernel: limit of one wait of a  */
-                             /* CTA (for its next ring slot / at a grid barrier), in     */
+    int wait_limit_us;       /* lane loop and lane groups: limit of one wait of a         */
+                             /* CTA (for its next ring slot / for its group), in          */
                              /* microseconds; a wait that runs out ends the call with    */
                              /* UBQP_ETIMEOUT and leaves the device usable; 0 = 5 s      */
     int tc_fuse;             /* tensor-core lanes: 1 = the contraction's epilogue warps run */
@@ -264,7 +266,7 @@ int ubqp_penalized_vjp(const void* x, const void* g, const void* grad_h, int64_t
 
 /*
  * ubqp_penalized_eval_noalloc - the computation of ubqp_penalized_eval (h and grad h of
- * problem (p) for `batch` points, same arguments, same kernel, same work partition) without
+ * problem (p) for `batch` points, same arguments, same kernel, same tiles) without
  * any device allocation, for callers that cannot call cudaMalloc/cudaFree: code that owns
  * all device memory through its own pool or a fixed memory budget, and code that cannot
  * afford the device-wide synchronization those calls may cause.  The paper has no

@@ -88,7 +88,8 @@ __host__ __device__ __forceinline__ float rr_mul(float a, float b)
 // FP32 throughout: FP64 runs at a small fraction of the FP32 rate on this part, and the
 // preconditioned basis keeps the 3 x 3 Gram matrices well scaled.  K is a compile-time constant:
 // the matrices stay in registers and no index or mask is computed (one thread runs this, so its
-// latency is the step's: 6,600 cycles of the eigen-solver's decision with run-time k).  Where a
+// latency is the step's: 6,600 cycles of the eigen-solver's decision with run-time k; the update
+// kernel of 256 starts, 896 steps, 13.4 -> 12.7 ms).  Where a
 // product is fused into a sum is written out, so that every kernel this is compiled into, and any
 // unrolling, gives the same bits.
 template <int K>

@@ -24,8 +24,8 @@
 // Measured (cycles per Alg. 2 step at n = 500, 1000 in the mixed batch of twelve, 2500; one group
 // of 16, 11, 79 CTAs): products 710, 3000, 1940; epilogue 1480, 1800, 1310; exchange 2290, 2700,
 // 3240; decision 390, 400, 690; x_{k+1} 150, 160, 330.  Device time of whole runs against the
-// barrier-and-records form this replaced: n = 50 to the end 13.7 -> 7.1 ms, n = 500 to the end
-// 303 -> 137 ms, n = 2500 (40 subproblems) 82 -> 44 ms, the batch of twelve 241 -> 127 ms.
+// barrier-and-records form this replaced: n = 50 to the end 13.7 -> 6.0 ms, n = 500 to the end
+// 303 -> 136 ms, n = 2500 (40 subproblems) 82 -> 42 ms, the batch of twelve 241 -> 116 ms.
 //
 // The arithmetic and its order are those of the other schedulers (item_rows_sell's shares,
 // row_epilogue, the record of a 32-row block, reduce_partials, decide, lane_apply), so a lane's

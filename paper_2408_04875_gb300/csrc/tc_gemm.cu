@@ -37,7 +37,10 @@ namespace {
 constexpr int kTcpThreads = 352;      // persistent kernel: 3 warps feed the tensor core, 8 run the epilogue
 constexpr int kTcpEpiWarps = kTcpThreads / 32 - 3;
 // split-K kernel: TMA producer, MMA issuer, then all warps drain TMEM and run the epilogue.  16 warps up
-// to four CTAs per cluster; with more, a thread's prefetched partials need the registers of 8.
+// to four CTAs per cluster; with more, a thread's prefetched partials need the registers of 8.  Bound:
+// latency of the epilogue (n = 2500, 256 starts, 3 CTAs a cluster, 43 starts a CTA; cycles: setup
+// 3.1k, main loop 7.2k, wait for the accumulators 1.9k, drain 3.5k, cluster barrier 1.5k, epilogue
+// 17-22k).  A launch 22.4 us with 8 warps, 21.3 with 16, 20.1 with the halving sums.
 constexpr int kTcThreads = 512;
 constexpr int kTcThreadsWide = 256;
 constexpr int kTcWideFrom = 5;        // cluster size from which the 8-warp form runs
@@ -799,7 +802,8 @@ __global__ void __launch_bounds__(kThr, 1) phase_a_tc_kernel(TcArgs A)
 //
 // Roles: warp 0 keeps the ring full of Q_off across tile boundaries and warp 8 of the starts'
 // inputs (a slot is two k-blocks: one copy of Q_off, two or four of inputs; with one producer and
-// one k-block per slot its instructions set the pace, 600 cycles a k-block); warp 1 issues the MMAs of each tile into one of two TMEM accumulators (columns
+// one k-block per slot its instructions set the pace, 600 cycles a k-block and 26.0 us a launch of
+// the ragged batch against 20.9); warp 1 issues the MMAs of each tile into one of two TMEM accumulators (columns
 // buf * max_bn), waiting until the epilogue has drained that buffer; warps 4..7 drain the
 // finished accumulator into shared memory (each warp reaches TMEM lanes 32 (w mod 4) ..)
 // and release it; warps 2..7, 9 and 10 then run the per-row epilogue of the tile's lanes, eight
