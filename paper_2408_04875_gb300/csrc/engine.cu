@@ -645,11 +645,14 @@ class Solver {
         for (int t = 0; t < ninst; ++t) row0[t + 1] = row0[t] + inst_[t].n;
         {
             std::vector<ValArgs> va(ninst);
+            int64_t pairs = 0;
             for (int t = 0; t < ninst; ++t) {
                 va[t].Q = inst_[t].Q;
                 va[t].b = inst_[t].b;
                 va[t].n = (int)inst_[t].n;
                 va[t].pad_ = 0;
+                va[t].pair0 = pairs;
+                pairs += validate_pairs(inst_[t].n);
                 va[t].out = ar_.at<float>(o_valid_) + 4 * t;
                 va[t].nnz = ar_.at<unsigned long long>(o_nnz_) + t;
             }
@@ -657,7 +660,7 @@ class Solver {
                                     cudaMemcpyHostToDevice, stream_));
             UBQP_CK(cudaMemcpyAsync(ar_.at<ValArgs>(o_valargs_), va.data(), va.size() * sizeof(ValArgs),
                                     cudaMemcpyHostToDevice, stream_));
-            UBQP_CK(launch_validate(ar_.at<ValArgs>(o_valargs_), ar_.at<int64_t>(o_row0_), ninst, row0[ninst], stream_));
+            UBQP_CK(launch_validate(ar_.at<ValArgs>(o_valargs_), ninst, pairs, stream_));
             launches_ += 1;
         }
         std::vector<float> val(insts.size() * 4);

@@ -81,37 +81,83 @@ __device__ __forceinline__ void atomic_max_nonneg(float* addr, float v)
     atomicMax(reinterpret_cast<int*>(addr), __float_as_int(v));  // v >= 0: int order = float order
 }
 
+constexpr int kValT = 64;   // validate: tile edge
+
 // out[0] = max |Q_ij - Q_ji|, out[1] = max |Q_ij| (i != j), out[2] = nonfinite flag, out[3] = max|Q|
-// and *nnz += the row's stored (nonzero) off-diagonal entries
-__device__ __forceinline__ void validate_row(const double* __restrict__ Q, const double* __restrict__ b, int n,
-                                             float* out, unsigned long long* nnz, int i)
+// and *nnz += the stored (nonzero) off-diagonal entries, over the pair of 64 x 64 tiles (I, J) and
+// (J, I) of Q.  Bound: reading Q once.  The tile below the diagonal goes through shared memory, so
+// that both are read along their rows (a row against its column took a 32-byte sector per entry of the
+// column), and a CTA adds its result once, a maximum only where it would raise it.  24 instances of
+// 100 to 3000 variables: 404 us a row at a time, 317 with FP64 comparisons, 198 with magnitudes as bits.
+__device__ __forceinline__ void validate_pair(const double* __restrict__ Q, const double* __restrict__ b, int n,
+                                              float* out, unsigned long long* nnz, int I, int J)
 {
-    __shared__ float sh[8];
-    float asym = 0.f, offmax = 0.f, qmax = 0.f, bad = 0.f;
-    unsigned cnt = 0;
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        double q = Q[(size_t)i * n + j];
-        double qt = Q[(size_t)j * n + i];
-        cnt += (j != i && q != 0.0) ? 1u : 0u;
-        if (!isfinite(q)) bad = 1.f;
-        float aq = (float)fabs(q);
-        qmax = fmaxf(qmax, aq);
-        if (j != i) offmax = fmaxf(offmax, aq);
-        double dq = fabs(q - qt);
-        asym = fmaxf(asym, isfinite(dq) ? (float)dq : 0.f);
+    __shared__ double st[kValT][kValT + 1];
+    __shared__ unsigned sh[8][5];
+    constexpr int kStep = 256 / kValT, kPer = kValT / kStep;
+    const int c = (int)threadIdx.x % kValT, r0 = (int)threadIdx.x / kValT;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool diag = I == J;
+    const int j = J * kValT + c, jt = I * kValT + c;   // columns of tiles (I, J) and (J, I)
+    double q[kPer];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        const int i = I * kValT + r0 + kStep * k;
+        q[k] = i < n && j < n ? Q[(size_t)i * n + j] : 0.0;
     }
-    if (threadIdx.x == 0 && b && !isfinite(b[i])) bad = 1.f;
-    for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-    if ((threadIdx.x & 31) == 0 && cnt) atomicAdd(nnz, (unsigned long long)cnt);
-    asym = block_max<256>(asym, sh);
-    offmax = block_max<256>(offmax, sh);
-    bad = block_max<256>(bad, sh);
-    qmax = block_max<256>(qmax, sh);
-    if (threadIdx.x == 0) {
-        atomic_max_nonneg(out + 0, asym);
-        atomic_max_nonneg(out + 1, offmax);
-        atomic_max_nonneg(out + 2, bad);
-        atomic_max_nonneg(out + 3, qmax);
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        const int i = J * kValT + r0 + kStep * k;
+        st[r0 + kStep * k][c] = diag ? q[k] : (i < n && jt < n ? Q[(size_t)i * n + jt] : 0.0);
+    }
+    __syncthreads();
+    // an entry past the edge is zero in both tiles and changes nothing.  Magnitudes are compared as bits
+    // (the float of the largest is the largest float): FP64 arithmetic only where the triangles differ
+    constexpr unsigned long long kInf = 0x7ff0000000000000ull;
+    unsigned long long top_off = 0, top_dia = 0;
+    float asym = 0.f;
+    bool bad = false;
+    unsigned cnt = 0;
+    auto entry = [&](unsigned long long mag, bool off) {
+        cnt += off && mag != 0 ? 1u : 0u;
+        bad |= mag >= kInf;
+        if (mag > kInf) return;   // NaN
+        if (off) top_off = mag > top_off ? mag : top_off;
+        else top_dia = mag > top_dia ? mag : top_dia;
+    };
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        const int r = r0 + kStep * k;
+        const double t = st[c][r];
+        const unsigned long long qb = (unsigned long long)__double_as_longlong(q[k]), tb = (unsigned long long)__double_as_longlong(t);
+        const bool off = !diag || r != c;
+        entry(qb & ~(1ull << 63), off);
+        if (!diag) entry(tb & ~(1ull << 63), true);
+        if (qb != tb) {
+            const double dq = fabs(q[k] - t);
+            asym = fmaxf(asym, isfinite(dq) ? (float)dq : 0.f);
+        }
+    }
+    const float offmax = (float)__longlong_as_double((long long)top_off);
+    const float qmax = fmaxf(offmax, (float)__longlong_as_double((long long)top_dia));
+    if (diag && b && r0 == 0 && j < n && !isfinite(b[j])) bad = true;
+    // nonnegative floats order as their bits
+    const unsigned w[5] = {__reduce_max_sync(0xffffffffu, __float_as_uint(asym)),
+                           __reduce_max_sync(0xffffffffu, __float_as_uint(offmax)),
+                           __reduce_max_sync(0xffffffffu, bad ? __float_as_uint(1.f) : 0u),
+                           __reduce_max_sync(0xffffffffu, __float_as_uint(qmax)), __reduce_add_sync(0xffffffffu, cnt)};
+    if (lane == 0)
+#pragma unroll
+        for (int a = 0; a < 5; ++a) sh[warp][a] = w[a];
+    __syncthreads();
+    if (threadIdx.x >= 5) return;
+    unsigned v = sh[0][threadIdx.x];
+#pragma unroll
+    for (int u = 1; u < 8; ++u) v = threadIdx.x == 4 ? v + sh[u][4] : max(v, sh[u][threadIdx.x]);
+    if (threadIdx.x == 4) {
+        if (v) atomicAdd(nnz, (unsigned long long)v);
+    } else if (__uint_as_float(v) > *reinterpret_cast<volatile float*>(out + threadIdx.x)) {
+        atomic_max_nonneg(out + threadIdx.x, __uint_as_float(v));
     }
 }
 
@@ -199,12 +245,21 @@ __device__ __forceinline__ int batch_instance(const int64_t* row0, int ninst, in
     return lo;
 }
 
-// every instance of a batch in one launch: one CTA per row of every instance
-__global__ void validate_kernel(const ValArgs* v, const int64_t* row0, int ninst)
+// every instance of a batch in one launch: one CTA per pair of tiles, the pairs I <= J of an instance
+// numbered down the columns (pair = J (J + 1) / 2 + I)
+__global__ void __launch_bounds__(256) validate_kernel(const ValArgs* v, int ninst)
 {
-    const int t = batch_instance(row0, ninst, blockIdx.x);
-    const ValArgs& a = v[t];
-    validate_row(a.Q, a.b, a.n, a.out, a.nnz, (int)(blockIdx.x - row0[t]));
+    int lo = 0, hi = ninst - 1;   // the last instance whose first pair is not past this one
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (v[mid].pair0 <= (int64_t)blockIdx.x) lo = mid; else hi = mid - 1;
+    }
+    const ValArgs& a = v[lo];
+    const int p = (int)((int64_t)blockIdx.x - a.pair0);
+    int J = (int)((sqrtf(8.f * (float)p + 1.f) - 1.f) * 0.5f);
+    while (J * (J + 1) / 2 > p) --J;
+    while ((J + 1) * (J + 2) / 2 <= p) ++J;
+    validate_pair(a.Q, a.b, a.n, a.out, a.nnz, p - J * (J + 1) / 2, J);
 }
 
 __global__ void reformulate_kernel(const RefArgs* args, const int64_t* row0, int ninst)
@@ -427,9 +482,15 @@ cudaError_t launch_pack_sym(const float* Qoff, int n, int ld, float* Qsym, cudaS
     return cudaGetLastError();
 }
 
-cudaError_t launch_validate(const ValArgs* v, const int64_t* row0, int ninst, int64_t rows, cudaStream_t s)
+int64_t validate_pairs(int64_t n)
 {
-    validate_kernel<<<(unsigned)rows, 256, 0, s>>>(v, row0, ninst);
+    const int64_t nb = (n + kValT - 1) / kValT;
+    return nb * (nb + 1) / 2;
+}
+
+cudaError_t launch_validate(const ValArgs* v, int ninst, int64_t pairs, cudaStream_t s)
+{
+    validate_kernel<<<(unsigned)pairs, 256, 0, s>>>(v, ninst);
     return cudaGetLastError();
 }
 

@@ -39,6 +39,7 @@ struct ValArgs {
     const double* b;
     float* out;
     unsigned long long* nnz;   // stored off-diagonal entries (nonzero Q_ij, i != j)
+    int64_t pair0;             // the instance's first pair of tiles in the launch
     int32_t n, pad_;
 };
 
@@ -69,7 +70,8 @@ struct FinalArgs {
 cudaError_t launch_pack_sym(const float* Qoff, int n, int ld, float* Qsym, cudaStream_t s);
 
 // one launch for every instance of a batch; row0[t] = first global row of instance t
-cudaError_t launch_validate(const ValArgs* v, const int64_t* row0, int ninst, int64_t rows, cudaStream_t s);
+int64_t validate_pairs(int64_t n);   // pairs of tiles of an n x n matrix
+cudaError_t launch_validate(const ValArgs* v, int ninst, int64_t pairs, cudaStream_t s);
 cudaError_t launch_reformulate(const RefArgs* args, const int64_t* row0, int ninst, int64_t rows, cudaStream_t s);
 cudaError_t launch_sell_width(const float* Qoff, int n, int ld, int32_t* width, cudaStream_t s);
 cudaError_t launch_sell_pack(const float* Qoff, int n, int ld, const int64_t* spo, float* vals, uint16_t* cols,
