@@ -247,12 +247,15 @@ __global__ void __launch_bounds__(kThreads, 2) grad_kernel(GradArgs A)
                 if (!isfinite(gi)) gi = 2.f * vf - 2.f * pi * xi + bi + pi;   // the pairs lose infinities
                 if (in && gp) *gp = gi;
                 const float th = __fmul_rn(xi, a);
-                float2 hs = make_float2(th, fmaf(xi, ae, fmaf(xi, a, -th)));
-                if (__any_sync(0xffffffffu, !isfinite(hs.x) || !isfinite(hs.y))) {
-                    hj = dsum_shfl_reduce((double)xi * ((double)vf + (double)bi + (double)pi - (double)pi * (double)xi));
-                } else {
-                    hs = csum_shfl_reduce(hs);
-                    hj = (double)hs.x + (double)hs.y;
+                const float2 h1 = make_float2(th, fmaf(xi, ae, fmaf(xi, a, -th)));
+                const float2 hs = csum_shfl_reduce(h1);
+                hj = (double)hs.x + (double)hs.y;
+                // FP64 where the pairs have left FP32's range: a share of h that is itself beyond it, or
+                // shares (finite ones) whose sums are, on the way or in the end
+                if (__any_sync(0xffffffffu, !isfinite(hj))) {
+                    const bool ok = isfinite(h1.x) && isfinite(h1.y);
+                    hj = dsum_shfl_reduce(ok ? (double)h1.x + (double)h1.y
+                                             : (double)xi * ((double)vf + (double)bi + (double)pi - (double)pi * (double)xi));
                 }
             } else {
                 const double* red = reinterpret_cast<const double*>(smem_raw) + j * kWarps * 32 + lane;
