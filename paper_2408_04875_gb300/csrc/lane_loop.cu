@@ -250,9 +250,8 @@ __global__ void __launch_bounds__(kThreads, 4) lane_loop_kernel(LoopArgs A)
 
 cudaError_t prepare_lane_loop(int max_ld)
 {
-    const size_t smem = (size_t)max_ld * sizeof(float);
     // always opted in: the static shared memory counts against the 48 KB default as well
-    return cudaFuncSetAttribute(lane_loop_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    return open_smem((const void*)lane_loop_kernel, (size_t)max_ld * sizeof(float));
 }
 
 // CTAs resident at once (the loop's CTAs wait on one another's pushes, so the grid never

@@ -742,19 +742,18 @@ static const void* sell_fn(int per)
 // the largest dynamic shared memory of a CTA when `per` (1 or 2) of them share an SM
 size_t sell_smem_limit(int per)
 {
-    int dev = 0, sm = 0, blk = 0, res = 0;
+    int dev = 0, sm = 0, res = 0;
+    size_t most = 0;
     cudaFuncAttributes fa;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&blk, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&res, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess ||
-        cudaFuncGetAttributes(&fa, sell_fn(per)) != cudaSuccess) {
+        cudaFuncGetAttributes(&fa, sell_fn(per)) != cudaSuccess || smem_limit(sell_fn(per), &most) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
     const int64_t a = (int64_t)sm / per - res - (int64_t)fa.sharedSizeBytes;
-    const int64_t b = (int64_t)blk - (int64_t)fa.sharedSizeBytes;
-    const int64_t v = std::min(a, b) / 1024 * 1024;
+    const int64_t v = std::min(a, (int64_t)most) / 1024 * 1024;
     return v > 0 ? (size_t)v : 0;
 }
 
@@ -762,7 +761,7 @@ size_t sell_smem_limit(int per)
 bool sell_fits(int per, size_t smem)
 {
     int got = 0;
-    if (cudaFuncSetAttribute(sell_fn(per), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+    if (open_smem(sell_fn(per), smem) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&got, sell_fn(per), kThreads, smem) != cudaSuccess) {
         cudaGetLastError();
         got = 0;

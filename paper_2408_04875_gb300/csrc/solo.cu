@@ -314,9 +314,8 @@ size_t solo_smem(int ld, bool one) { return (one ? 6 : 2) * (size_t)ld * sizeof(
 
 cudaError_t prepare_solo(int ld, bool one)
 {
-    const size_t smem = solo_smem(ld, one);
     // always opted in: the static shared memory counts against the 48 KB default as well
-    return cudaFuncSetAttribute(solo_lane_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    return open_smem((const void*)solo_lane_kernel, solo_smem(ld, one));
 }
 
 // CTAs of the kernel resident on one SM with the dynamic shared memory of lanes of ld

@@ -647,21 +647,18 @@ size_t sym_lane_words(int nb)
 // 0 when even those vectors do not fit.  mat_bytes: the tiles' part
 size_t sym_lane_smem(int ld, int tiles, int32_t* mat_bytes)
 {
-    int dev = 0, blk = 0;
-    cudaFuncAttributes fa;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&blk, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
-        cudaFuncGetAttributes(&fa, sym_lane_kernel) != cudaSuccess) {
+    size_t most = 0;
+    if (smem_limit((const void*)sym_lane_kernel, &most) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
     const int64_t base = 2 * (int64_t)ld * 4 + (int64_t)(ld / kSymT) * kBlkRows * 4;
-    const int64_t room = (int64_t)blk - (int64_t)fa.sharedSizeBytes - base;
+    const int64_t room = (int64_t)most - base;
     if (room < 0) return 0;
     const int64_t fit = std::min<int64_t>(tiles, room / kTileBytes);
     *mat_bytes = (int32_t)(fit * kTileBytes);
     const size_t smem = (size_t)(base + fit * kTileBytes);
-    if (cudaFuncSetAttribute(sym_lane_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    if (open_smem((const void*)sym_lane_kernel, smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }

@@ -1143,7 +1143,7 @@ int tcp_grid(const TcArgs& a, int ntiles)
     int dev = 0, sms = 148, per = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaFuncSetAttribute(phase_a_tcp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+    if (open_smem((const void*)phase_a_tcp_kernel, smem) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, phase_a_tcp_kernel, kTcpThreads, smem) != cudaSuccess ||
         per < 1) {
         cudaGetLastError();
@@ -1156,7 +1156,7 @@ int tcp_grid(const TcArgs& a, int ntiles)
 cudaError_t tcp_launch(const TcArgs& a, int ntiles, int grid, cudaStream_t st)
 {
     const size_t smem = tcp_smem_bytes(a.max_bn, a.two_any != 0, a.kbs, a.stages);
-    cudaError_t e = cudaFuncSetAttribute(phase_a_tcp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = open_smem((const void*)phase_a_tcp_kernel, smem);
     if (e != cudaSuccess) return e;
     phase_a_tcp_kernel<<<grid, kTcpThreads, smem, st>>>(a, ntiles);
     return cudaGetLastError();
@@ -1188,7 +1188,7 @@ cudaError_t tc_launch(const TcArgs& a, int total_clusters, int S, cudaStream_t s
 {
     const size_t smem = tc_smem_bytes(a.max_bn, a.two_any != 0, a.stages);
     const TcKernel k = tc_kernel(S);
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = open_smem((const void*)k, smem);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = tc_config(total_clusters * S, S, smem, attr);
@@ -1200,7 +1200,7 @@ int tc_max_active_clusters(int bn, bool two, int stages, int S)
 {
     const size_t smem = tc_smem_bytes(bn, two, stages);
     const TcKernel k = tc_kernel(S);
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
+    if (open_smem((const void*)k, smem) != cudaSuccess) return 0;
     cudaLaunchAttribute attr[1];
     const cudaLaunchConfig_t cfg = tc_config(S * 64, S, smem, attr);
     int n = 0;

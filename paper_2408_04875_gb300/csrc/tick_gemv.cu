@@ -69,8 +69,7 @@ __global__ void __launch_bounds__(kThreads, 4) phase_a_gemv_kernel(TickArgs A)
 cudaError_t prepare_phase_a_gemv(int max_ld)
 {
     // always opted in: the static shared memory counts against the 48 KB default as well
-    return cudaFuncSetAttribute(phase_a_gemv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)((size_t)max_ld * sizeof(float)));
+    return open_smem((const void*)phase_a_gemv_kernel, (size_t)max_ld * sizeof(float));
 }
 
 // persistent grid: every CTA that fits on the GPU at once, never more CTAs than items

@@ -543,6 +543,13 @@ cudaError_t work_alloc(void** p, size_t bytes, cudaStream_t s);
 cudaError_t pinned_get(void** p);   // 64 bytes
 void pinned_put(void* p);
 
+// Dynamic shared memory.  A kernel's limit is one number for the whole process, so it is always set
+// to the most a launch can have, never to one call's size: a second host thread with a smaller
+// problem would otherwise lower it between the first thread's launches.  open_smem fails when a launch
+// of `need` bytes could not run; smem_limit gives the most (workspace.cu).
+cudaError_t smem_limit(const void* kernel, size_t* bytes);
+cudaError_t open_smem(const void* kernel, size_t need);
+
 // the calling thread's last-error text (ubqp_last_error), shared by every entry point
 void set_error(const char* fmt, ...);
 void clear_error();

@@ -136,6 +136,28 @@ cudaError_t pinned_get(void** p)
     return cudaMallocHost(p, kPinnedBytes);
 }
 
+cudaError_t smem_limit(const void* kernel, size_t* bytes)
+{
+    int dev = 0, blk = 0;
+    cudaFuncAttributes fa;
+    *bytes = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&blk, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kernel);
+    if (e != cudaSuccess) return e;
+    if ((size_t)blk > fa.sharedSizeBytes) *bytes = (size_t)blk - fa.sharedSizeBytes;
+    return cudaSuccess;
+}
+
+cudaError_t open_smem(const void* kernel, size_t need)
+{
+    size_t most = 0;
+    cudaError_t e = smem_limit(kernel, &most);
+    if (e != cudaSuccess) return e;
+    if (need > most) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 void pinned_put(void* p)
 {
     unsigned long long id = 0;
