@@ -331,6 +331,19 @@ int ubqp_initial_point(const double* Q, const double* b, const double* mu, int64
 int64_t ubqp_profile_timeline(float* ms_out, int64_t* work_out, int64_t cap);
 
 /*
+ * ubqp_profile_groups - the plan of the first launch of the last call on this thread that ran
+ * its lanes on groups of CTAs (stats.gemv_kernel = 3).  Writes up to `cap` of these into out:
+ *   [0] the kernel: 1 sliced rows (sell_lane_kernel), 2 symmetric tiles (sym_lane_kernel),
+ *       3 group barriers on any storage (solo_lane_kernel)
+ *   [1] CTAs that share an SM
+ *   [2] the most row blocks (kernel 2: tiles) a CTA owns
+ *   [3] bytes of matrix entries a CTA keeps in shared memory (kernel 3: 0)
+ *   [4] CTAs of the launch
+ * and returns how many there are (5), or 0 when no call on this thread used groups.
+ */
+int32_t ubqp_profile_groups(int32_t* out, int32_t cap);
+
+/*
  * ubqp_tc_matmul_probe - test entry: the tensor-core contraction of the batched path on
  * its own, D = A (B_hi + B_lo)^T with FP32 accumulation, returned raw.
  *   A n x n, B_hi and B_lo (B_lo may be NULL) R x n, all BF16 bit patterns in HOST memory,

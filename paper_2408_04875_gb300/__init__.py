@@ -96,6 +96,8 @@ def lib():
             L.ubqp_penalty_probe.argtypes = [vp, vp, vp, vp, i64, C.POINTER(Opts), C.POINTER(C.c_double),
                                              C.POINTER(C.c_double), C.POINTER(i32), C.POINTER(i32)]
             L.ubqp_initial_point.argtypes = [vp, vp, vp, i64, C.POINTER(Opts), vp, vp]
+            L.ubqp_profile_groups.restype = i32
+            L.ubqp_profile_groups.argtypes = [vp, i32]
             for name in ("ubqp_solve", "ubqp_solve_batched", "ubqp_penalized_eval", "ubqp_penalized_vjp",
                          "ubqp_penalized_eval_noalloc", "ubqp_inner_run", "ubqp_penalty_probe",
                          "ubqp_initial_point"):
@@ -189,6 +191,19 @@ def solve_batched(Qs, bs=None, mus=None, starts=None, **kw):
     d = st.as_dict()
     d["status"] = rc
     return xs, obj, d
+
+
+GROUP_KERNELS = {1: "sell_lane_kernel", 2: "sym_lane_kernel", 3: "solo_lane_kernel"}
+
+
+def lane_groups():
+    """The plan of the last call on this thread that ran its lanes on groups of CTAs (its first
+    launch): the kernel, CTAs per SM, the most row blocks or tiles of a CTA, the bytes of matrix
+    entries a CTA keeps in shared memory, and the CTAs.  None before any such call."""
+    v = (C.c_int32 * 5)()
+    if lib().ubqp_profile_groups(v, 5) == 0:
+        return None
+    return {"kernel": GROUP_KERNELS[v[0]], "ctas_per_sm": v[1], "blocks_per_cta": v[2], "smem_bytes": v[3], "ctas": v[4]}
 
 
 def solve(Q, b=None, mu=None, starts=None, **kw):

@@ -28,6 +28,7 @@
 namespace ubqp {
 
 static thread_local char g_last_error[512] = "";
+static thread_local int32_t g_groups[5] = {0, 0, 0, 0, 0};   // ubqp_profile_groups
 static thread_local std::vector<float> g_tl_ms;
 static thread_local std::vector<int64_t> g_tl_work;
 
@@ -1300,6 +1301,17 @@ class Solver {
             if (plan_solo_groups(ids, max_ld_, true)) UBQP_CK(upload_solo_plan());
         }
         set_plan();
+        {
+            int32_t most = symg_ ? sym_group_tiles() : 1;
+            for (size_t g = 0; !symg_ && g + 1 < solo_gcta_.size(); ++g)
+                for (int q = solo_gfirst_[g]; q < solo_gfirst_[g + 1]; ++q) {
+                    const int nc = solo_gcta_[g + 1] - solo_gcta_[g];
+                    most = std::max(most, (lanes_[(size_t)solo_glanes_[q]].nblk + nc - 1) / nc);
+                }
+            const int32_t r[5] = {symg_ ? 2 : (sell_ ? 1 : 3), symg_ ? 1 : solo_per_, most,
+                                  symg_ || sell_ ? sa.mat_bytes : 0, sa.grid};
+            std::copy(r, r + 5, g_groups);
+        }
         sa.rows_per_item = rows_per_item_;
         sa.budget = probe_ticks_ > 0 ? probe_ticks_ : (o_.lane_budget > 0 ? o_.lane_budget : 1024);
         int32_t* ctl = ar_.at<int32_t>(o_solo_);
@@ -1946,6 +1958,13 @@ int64_t ubqp_profile_timeline(float* ms_out, int64_t* work_out, int64_t cap)
         if (work_out) work_out[i] = g_tl_work[(size_t)i];
     }
     return n;
+}
+
+int32_t ubqp_profile_groups(int32_t* out, int32_t cap)
+{
+    if (g_groups[0] == 0) return 0;
+    for (int32_t i = 0; i < 5 && i < cap; ++i) out[i] = g_groups[i];
+    return 5;
 }
 
 // every instance's R lanes: start 0 from x^0 of Eq. (gamma) (Jacobi sweeps first), the

@@ -1,0 +1,57 @@
+"""Which kernel runs the lane groups, and with which plan: ubqp_profile_groups after calls whose
+results other tests compare (the kernels give the same bits, so a call that silently ran another one
+would pass those)."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ub():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    import paper_2408_04875_gb300 as m
+    return m
+
+
+def _plan(ub, sizes, density, **kw):
+    from paper_2408_04875_gb300 import instances as I
+    Qs = [I.random_ubqp(n, density, k)[0] for k, n in enumerate(sizes)]
+    _, _, st = ub.solve_batched(Qs, None, max_outer=2, max_inner=20, seed=1, **kw)
+    assert st["gemv_kernel"] == 3
+    return ub.lane_groups(), [int((Q != 0).sum(1).max()) for Q in Qs]
+
+
+def test_one_sparse_lane(ub):
+    for n, ctas in ((40, 1), (256, 1), (257, 9), (2500, 79)):
+        g, width = _plan(ub, (n,), 0.1)
+        assert (g["kernel"], g["ctas_per_sm"], g["blocks_per_cta"], g["ctas"]) == ("sell_lane_kernel", 1, 1, ctas)
+        assert g["smem_bytes"] > 0
+
+
+def test_slices_that_fit_and_slices_that_do_not(ub):
+    # 192 bytes (32 entries of six) per column of a slice's widest row
+    g, width = _plan(ub, (2500, 2500, 2500, 1000, 1000, 250, 250), 0.1)
+    assert g["kernel"] == "sell_lane_kernel" and g["blocks_per_cta"] > 1
+    assert g["smem_bytes"] >= 192 * (max(width) - 1)
+    g, width = _plan(ub, (1500, 1400, 1300, 1500, 1200, 1500, 1450, 1350), 0.3)
+    assert g["kernel"] == "sell_lane_kernel"
+    assert g["smem_bytes"] < g["blocks_per_cta"] * 192 * (max(width) - 1)
+
+
+def test_two_ctas_per_sm(ub):
+    g, width = _plan(ub, (1100,) * 24, 0.1)
+    assert (g["kernel"], g["ctas_per_sm"], g["blocks_per_cta"]) == ("sell_lane_kernel", 2, 3)
+    assert g["smem_bytes"] < 3 * 192 * (max(width) - 1)   # not all of a CTA's slices
+    g, _ = _plan(ub, (600,) * 20, 0.1)
+    assert (g["kernel"], g["ctas_per_sm"]) == ("sell_lane_kernel", 1)
+
+
+def test_dense_lanes(ub):
+    g, _ = _plan(ub, (1000, 900, 1000, 800), 0.7)
+    assert g["kernel"] == "sym_lane_kernel" and g["smem_bytes"] == g["blocks_per_cta"] * 65536
+    g, _ = _plan(ub, (1000,), 0.7)
+    assert g["kernel"] == "solo_lane_kernel"
+    g, _ = _plan(ub, (1000,), 0.1, rows_per_item=64)
+    assert g["kernel"] == "solo_lane_kernel"
