@@ -1318,9 +1318,9 @@ class Solver {
         sa.err = ctl;
         sa.active_after = ctl + 1;
         sa.bar = reinterpret_cast<unsigned*>(ctl + 4);
-        sa.wait_ns = o_.wait_limit_us > 0 ? 1000ull * (unsigned long long)o_.wait_limit_us : 5000000000ull;
+        const unsigned long long wait_us = o_.wait_limit_us > 0 ? (unsigned long long)o_.wait_limit_us : 5000000ull;
         // (the highest SM clock is 2070 MHz; asking the runtime for it takes 600 us)
-        sa.wait_cycles = sa.wait_ns / 1000ull * 2100ull;
+        sa.wait_cycles = wait_us * 2100ull;
         sa.fast = 1;
         sa.one_ok = solo_one_ok_ ? 1 : 0;
         sa.P = make_params(o_, ar_.at<int64_t>(o_hist_));
@@ -1355,7 +1355,8 @@ class Solver {
                 phase_a_launches_ += 1;
             }
             if (h_active_[0]) {
-                set_error("a bounded wait in the single-lane kernel ran out (limit %.0f us)", (double)sa.wait_ns * 1e-3);
+                set_error("a bounded wait in the lane-group or single-lane kernel (%s) ran out (limit %llu us)",
+                          symg_ ? "sym_lane_kernel" : (sell_ ? "sell_lane_kernel" : "solo_lane_kernel"), wait_us);
                 return UBQP_ETIMEOUT;
             }
             if (probe_ticks_ > 0) break;

@@ -494,10 +494,10 @@ struct SoloArgs {
     unsigned* bar;              // per group (stride kSoloBarStride words): a 64-bit arrival counter
     int32_t* err;               // set when a bounded wait runs out
     int32_t* active_after;      // lanes unfinished at the end of the launch (the caller zeroes it)
-    unsigned long long wait_ns; // limit of one wait of a CTA for the others of its group ...
-    unsigned long long wait_cycles;   // ... in SM cycles (at the highest SM clock, so never shorter);
-                                // the waits read the SM's own counter: reading the global timer
-                                // takes longer than the wait it would bound
+    unsigned long long wait_cycles;   // limit of one wait of a CTA for the others of its group, in SM
+                                // cycles (at the highest SM clock, so never shorter); the waits read the
+                                // SM's own counter: reading the global timer takes longer than the wait
+                                // it would bound
     int32_t fast;               // Alg. 2 steps with one barrier (whole x_k in every CTA)
     int32_t one_ok;             // shared memory holds the one-CTA state (6 vectors)
     int32_t mat_bytes;          // sell_lane.cu, sym_lane.cu: shared memory of a CTA for its entries / tiles
