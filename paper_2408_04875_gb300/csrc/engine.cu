@@ -1341,7 +1341,7 @@ class Solver {
             UBQP_CK(cudaMemsetAsync(sa.active_after, 0, sizeof(int32_t), stream_));
             if (prof) UBQP_CK(cudaEventRecord(evA_[0], stream_));
             if (symg_) UBQP_CK(launch_sym(sa, sell_smem_, stream_));
-            else if (sell_) UBQP_CK(launch_sell(sa, solo_per_, sell_smem_, stream_));
+            else if (sell_) UBQP_CK(launch_sell(sa, solo_per_, sell_tight_, sell_smem_, stream_));
             else UBQP_CK(launch_solo(sa, max_ld_, stream_));
             if (prof) UBQP_CK(cudaEventRecord(evA_[1], stream_));
             UBQP_CK(cudaMemcpyAsync(h_active_, ctl, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, stream_));
@@ -1517,14 +1517,17 @@ class Solver {
         int w = 0;
         for (int l : ids) w = std::max(w, inst_[(size_t)lane_inst_[l]].max_width);
         if (m > kSoloMaxSl || w == 0 || rows_per_item_ != 32) return 1e9 + 1e3 * m + per;   // solo.cu: the smallest m
-        const int64_t room = (int64_t)sell_smem_limit(per) - 2 * (int64_t)max_ld * (int64_t)sizeof(float);
+        bool tight;
+        const size_t vecs = 2 * (size_t)max_ld * sizeof(float);
+        const int64_t room = (int64_t)sell_smem_limit(per, vecs, &tight) - (int64_t)vecs;
+        if (room < 0) return 1e9 + 1e3 * m + per;   // the vectors do not fit: solo.cu
         const int64_t res = std::max<int64_t>(0, std::min<int64_t>(m, room / (192 * (int64_t)w)));
         return per * w * (3.5 * (double)res + 17.5 * (double)(m - res));
     }
 
     // Whether the current plan runs on the sliced kernel (sell_lane.cu), and its shared memory:
     // two vectors and as many of a CTA's slices as fit
-    bool sell_shape(size_t* smem, int32_t* mat_bytes) const
+    bool sell_shape(size_t* smem, int32_t* mat_bytes)
     {
         if (!sparse_) return false;
         size_t mat = 0;
@@ -1537,12 +1540,13 @@ class Solver {
                 const size_t slices = one ? (size_t)(L.n + 31) / 32 : (size_t)((L.nblk + nc - 1) / nc);
                 mat = std::max(mat, slices * (size_t)inst_[(size_t)lane_inst_[solo_glanes_[q]]].max_width * 192);
             }
-        const size_t limit = sell_smem_limit(solo_per_), vecs = 2 * (size_t)max_ld_ * sizeof(float);
+        if (solo_per_ > 2) return false;
+        const size_t vecs = 2 * (size_t)max_ld_ * sizeof(float), limit = sell_smem_limit(solo_per_, vecs, &sell_tight_);
         if (vecs > limit) return false;
         mat = std::min(mat, limit - vecs);
         *smem = vecs + mat;
         *mat_bytes = (int32_t)mat;
-        return solo_per_ <= 2 && sell_fits(solo_per_, *smem);
+        return sell_fits(solo_per_, sell_tight_, *smem);
     }
 
     // the group tables to the device (glanes, then gfirst and gcta at fixed offsets) and the
@@ -1839,7 +1843,8 @@ class Solver {
     int solo_max_lanes_ = 1;
     int64_t solo_capc_ = 0;      // CTAs resident at once
     int solo_per_ = 1;           // CTAs of the current plan that share an SM
-    bool sell_ = false;          // the current plan runs on the sliced kernel
+    bool sell_ = false;          // the current plan runs on the sliced kernel ...
+    bool sell_tight_ = false;    // ... in its tight form
     bool symg_ = false;          // groups of CTAs on the symmetric tiles
     size_t sell_smem_ = 0;
     size_t solo_gmax_ = 1;       // groups the tables and barriers have room for

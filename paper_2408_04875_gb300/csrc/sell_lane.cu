@@ -155,12 +155,17 @@ struct __align__(16) ShareAt {
 
 }  // namespace
 
-// kPer CTAs share an SM (1: up to 255 registers a thread; 2: 128)
-template <int kPer>
+// kPer CTAs share an SM (1: up to 255 registers a thread; 2: 128).  kTight: what the owner of a slice
+// leaves for the other warps (the eigen-solver's vectors at its 32 rows, or the rows' products in FP64)
+// lies over the slice's shares, which the owner has read by then, instead of in 8 KB of its own.  Two CTAs
+// on an SM then hold vectors up to ld = 12,416 instead of 11,392; shorter ones keep the other form,
+// which is up to 1.5 % faster on lanes of one CTA.  Three and four lanes of n = 12000, density 0.002,
+// two subproblems, device time: 5.0 and 5.7 ms, against 7.8 and 8.8 ms on solo.cu.
+template <int kPer, bool kTight>
 __global__ void __launch_bounds__(kThreads, kPer) sell_lane_kernel(SoloArgs A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ double sv[kThreads];
+    __shared__ double s_sv[kTight ? 1 : kThreads];
     __shared__ LaneState S;
     __shared__ Partial R;
     __shared__ Decision D;
@@ -169,7 +174,7 @@ __global__ void __launch_bounds__(kThreads, kPer) sell_lane_kernel(SoloArgs A)
     __shared__ float2 s_share[kSoloMaxSl * kThreads];
     __shared__ WarpRed s_red[kWarps];
     __shared__ WarpRed s_rec[kSoloMaxSl];   // records of a one-CTA group
-    __shared__ float s_basis[kWarps][6 * 32];   // the eigen-solver's vectors at the CTA's rows
+    __shared__ float s_basis[kTight ? 1 : kWarps][6 * 32];   // the eigen-solver's vectors at the CTA's rows
     __shared__ SliceAt s_sl[kWarps];
     __shared__ ShareAt s_sh[kWarps][kWarps];
     __shared__ __align__(16) LaneDev sL;
@@ -273,6 +278,19 @@ __global__ void __launch_bounds__(kThreads, kPer) sell_lane_kernel(SoloArgs A)
         const bool own = own_warp && row < n;
         const int rc = own ? row : n - 1;
         const float2* my_sh = s_share + (one ? warp * wps * 32 : warp * kThreads) + lane;   // share p at 32 p
+
+        // where the owner of slice b leaves its vectors and its rows' products.  A lane of one block has its
+        // shares in the first kThreads entries of s_share and the rest free.
+        constexpr int kOwn = 6 * 32 / 2;   // float2 entries
+        static_assert(kThreads + kWarps * kOwn <= kSoloMaxSl * kThreads && kOwn <= kThreads, "room for what the owners leave");
+        auto basis = [&](int b) -> float* {
+            if constexpr (kTight) return reinterpret_cast<float*>(s_share + (one ? kThreads + b * kOwn : b * kThreads));
+            else return s_basis[b];
+        };
+        auto prods = [&](int b) -> double* {
+            if constexpr (kTight) return reinterpret_cast<double*>(s_share + (one ? kThreads + b * 32 : b * kThreads));
+            else return s_sv + 32 * b;
+        };
 
         // the products of every slice of this CTA, shares into s_share; then v of the own row
         auto share = [&](int b, int part) -> float2 {
@@ -555,7 +573,8 @@ __global__ void __launch_bounds__(kThreads, kPer) sell_lane_kernel(SoloArgs A)
                     if (own_warp) {
                         const float v = own_product();
                         if (own && r_d != 0.f) aw = r_d * fmaf(r_dmp, r_d * lw, v);
-                        float* q = s_basis[warp] + lane;   // rows beyond n hold zeros
+                        if constexpr (kTight) __syncwarp();   // the shares are read
+                        float* q = basis(warp) + lane;   // rows beyond n hold zeros
                         q[0] = lx;
                         q[32] = lax;
                         q[64] = lw;
@@ -568,7 +587,7 @@ __global__ void __launch_bounds__(kThreads, kPer) sell_lane_kernel(SoloArgs A)
                     // ---- the twelve Gram sums of every slice, two per warp and turn
                     for (int task = warp; task < 6 * sl.n; task += kWarps) {
                         const int b = task / 6, t = 2 * (task - 6 * b);
-                        const float* q = s_basis[b] + lane;
+                        const float* q = basis(b) + lane;
                         float2 s[2];
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
@@ -687,6 +706,7 @@ __global__ void __launch_bounds__(kThreads, kPer) sell_lane_kernel(SoloArgs A)
                 item_load_u(L, su);
                 __syncthreads();
                 if (ph == PH_EVAL) {
+                    double* sv = kTight ? reinterpret_cast<double*>(s_share) : s_sv;
                     for (int blk = rank; blk < nblk; blk += nc) {
                         const int row0 = blk * A.rows_per_item;
                         const int rows = min(A.rows_per_item, n - row0);
@@ -699,11 +719,19 @@ __global__ void __launch_bounds__(kThreads, kPer) sell_lane_kernel(SoloArgs A)
                     // the products of all slices first, then the blocks' epilogues
                     products();
                     __syncthreads();
-                    if (own_warp) sv[tid] = (double)own_product();
+                    if constexpr (kTight) {
+                        if (own_warp) {
+                            const float v = own_product();
+                            __syncwarp();   // the shares are read
+                            prods(warp)[lane] = (double)v;
+                        }
+                    } else if (own_warp) {
+                        s_sv[tid] = (double)own_product();
+                    }
                     __syncthreads();
                     for (int b = 0; b < (one ? 1 : sl.n); ++b) {
                         const int blk = one ? 0 : sl.at(b), row0 = 32 * blk;
-                        item_finish(L, ph, S.k, blk, row0, one ? n : min(32, n - row0), sv + 32 * b, P);
+                        item_finish(L, ph, S.k, blk, row0, one ? n : min(32, n - row0), prods(b), P);
                         __syncthreads();
                     }
                 }
@@ -734,13 +762,13 @@ __global__ void __launch_bounds__(kThreads, kPer) sell_lane_kernel(SoloArgs A)
     }
 }
 
-static const void* sell_fn(int per)
+static const void* sell_fn(int per, bool tight)
 {
-    return per == 1 ? (const void*)sell_lane_kernel<1> : (const void*)sell_lane_kernel<2>;
+    if (per == 1) return (const void*)sell_lane_kernel<1, false>;
+    return tight ? (const void*)sell_lane_kernel<2, true> : (const void*)sell_lane_kernel<2, false>;
 }
 
-// the largest dynamic shared memory of a CTA when `per` (1 or 2) of them share an SM
-size_t sell_smem_limit(int per)
+static size_t sell_limit(const void* fn, int per)
 {
     int dev = 0, sm = 0, res = 0;
     size_t most = 0;
@@ -748,7 +776,7 @@ size_t sell_smem_limit(int per)
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&res, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess ||
-        cudaFuncGetAttributes(&fa, sell_fn(per)) != cudaSuccess || smem_limit(sell_fn(per), &most) != cudaSuccess) {
+        cudaFuncGetAttributes(&fa, fn) != cudaSuccess || smem_limit(fn, &most) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -757,23 +785,35 @@ size_t sell_smem_limit(int per)
     return v > 0 ? (size_t)v : 0;
 }
 
+// the largest dynamic shared memory of a CTA when `per` (1 or 2) of them share an SM and `vecs` bytes
+// of it are vectors: the tight form where the other does not hold them
+size_t sell_smem_limit(int per, size_t vecs, bool* tight)
+{
+    *tight = false;
+    const size_t v = sell_limit(sell_fn(per, false), per);
+    if (per == 1 || vecs <= v) return v;
+    *tight = true;
+    return sell_limit(sell_fn(per, true), per);
+}
+
 // whether `per` CTAs with this much dynamic shared memory are resident on an SM
-bool sell_fits(int per, size_t smem)
+bool sell_fits(int per, bool tight, size_t smem)
 {
     int got = 0;
-    if (open_smem(sell_fn(per), smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&got, sell_fn(per), kThreads, smem) != cudaSuccess) {
+    const void* fn = sell_fn(per, tight);
+    if (open_smem(fn, smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&got, fn, kThreads, smem) != cudaSuccess) {
         cudaGetLastError();
         got = 0;
     }
     return got >= per;
 }
 
-cudaError_t launch_sell(const SoloArgs& a, int per, size_t smem, cudaStream_t s)
+cudaError_t launch_sell(const SoloArgs& a, int per, bool tight, size_t smem, cudaStream_t s)
 {
     SoloArgs args = a;
     void* params[] = {&args};
-    return cudaLaunchCooperativeKernel(sell_fn(per), dim3((unsigned)a.grid), dim3(kThreads), params, smem, s);
+    return cudaLaunchCooperativeKernel(sell_fn(per, tight), dim3((unsigned)a.grid), dim3(kThreads), params, smem, s);
 }
 
 }  // namespace ubqp

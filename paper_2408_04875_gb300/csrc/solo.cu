@@ -21,7 +21,8 @@
 // and computes step k+1 never overwrites g_k or a record of step k that another CTA of the
 // group may still be reading.  When the subproblem ends, or the launch's budget does, the CTAs write x_k,
 // x_{k-1} and u back.  Lanes on the sliced storage run sell_lane.cu instead, except those whose
-// blocks are not 32 rows or whose CTAs own more than kSoloMaxSl slices.  The arithmetic is that
+// blocks are not 32 rows, whose CTAs own more than kSoloMaxSl slices, or whose two vectors leave that
+// kernel no room (two CTAs per SM, ld > 12,416).  The arithmetic is that
 // of the lock-step scheduler with the same rows per item, so both give the same bits.  Every
 // group barrier wait is bounded: when it runs out the CTA sets the error flag and leaves, and
 // the others leave at their own next wait.  A group of one CTA needs no barrier.

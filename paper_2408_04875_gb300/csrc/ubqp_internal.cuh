@@ -515,9 +515,9 @@ cudaError_t launch_solo(const SoloArgs& a, int ld, cudaStream_t s);
 // the same groups on the sliced storage, at most kSoloMaxSl slices per CTA (or a lane of one block
 // on one CTA): entries in shared memory, one-hop exchanges (sell_lane.cu)
 constexpr int kSellWordsPerBlock = 74;   // 16-byte exchange words per row block, two buffers
-size_t sell_smem_limit(int per);
-bool sell_fits(int per, size_t smem);
-cudaError_t launch_sell(const SoloArgs& a, int per, size_t smem, cudaStream_t s);
+size_t sell_smem_limit(int per, size_t vecs, bool* tight);
+bool sell_fits(int per, bool tight, size_t smem);
+cudaError_t launch_sell(const SoloArgs& a, int per, bool tight, size_t smem, cudaStream_t s);
 
 // the same groups on the symmetric tiles, at most kSymMaxTiles tiles per CTA (sym_lane.cu)
 constexpr int kSymMaxTiles = 20;

@@ -41,7 +41,7 @@ def test_slices_that_fit_and_slices_that_do_not(ub):
 
 
 def test_two_ctas_per_sm(ub):
-    g, width = _plan(ub, (1100,) * 24, 0.1)
+    g, width = _plan(ub, (1100,) * 24, 0.15)
     assert (g["kernel"], g["ctas_per_sm"], g["blocks_per_cta"]) == ("sell_lane_kernel", 2, 3)
     assert g["smem_bytes"] < 3 * 192 * (max(width) - 1)   # not all of a CTA's slices
     g, _ = _plan(ub, (600,) * 20, 0.1)
@@ -55,3 +55,28 @@ def test_dense_lanes(ub):
     assert g["kernel"] == "solo_lane_kernel"
     g, _ = _plan(ub, (1000,), 0.1, rows_per_item=64)
     assert g["kernel"] == "solo_lane_kernel"
+
+
+# two CTAs on an SM hold two vectors of up to 12,416 entries: three lanes of 11,600 and 12,320 need more than five
+# slices per CTA with one CTA per SM, and run on the sliced kernel with two, with the bits of the lock-step
+# scheduler
+@pytest.mark.parametrize("n", [11600, 12320])
+def test_long_vectors_on_two_ctas_per_sm(ub, n):
+    import torch
+    Qs = []
+    for k in range(3):
+        g = torch.Generator(device="cuda").manual_seed(k)
+        v = torch.randint(-100, 101, (n, n), generator=g, device="cuda").double()
+        v *= torch.rand(n, n, generator=g, device="cuda") < 0.002
+        u = torch.triu(v)
+        Qs.append((u + torch.triu(v, 1).T).contiguous())
+        del v, u
+    kw = dict(max_outer=2, max_inner=30, seed=1)
+    xs, f, st = ub.solve_batched(Qs, None, lane_budget=40, **kw)
+    g = ub.lane_groups()
+    assert st["gemv_kernel"] == 3
+    assert (g["kernel"], g["ctas_per_sm"], g["blocks_per_cta"]) == ("sell_lane_kernel", 2, 4)
+    ys, h, ref = ub.solve_batched(Qs, None, gemv_kernel=1, rows_per_item=32, **kw)
+    assert (f == h).all() and all((x == y).all() for x, y in zip(xs, ys))
+    for k in ("inner_steps", "inner_iters", "outer_steps", "lobpcg_iters", "jacobi_iters", "floor_steps"):
+        assert st[k] == ref[k], k
