@@ -278,9 +278,10 @@ class Solver {
         if (ev1_) cudaEventDestroy(ev1_);
         for (auto e : evA_) cudaEventDestroy(e);
         if (stream_) {
-            cudaStreamSynchronize(stream_);
             ar_.release();
             sp_ar_.release();
+            // also gives back what the pool holds beyond its limit, before the call returns
+            cudaStreamSynchronize(stream_);
             cudaStreamDestroy(stream_);
         }
     }
