@@ -37,7 +37,10 @@ namespace {
 constexpr int kTcpThreads = 352;      // persistent kernel: 3 warps feed the tensor core, 8 run the epilogue
 constexpr int kTcpEpiWarps = kTcpThreads / 32 - 3;
 // split-K kernel: TMA producer, MMA issuer, then all warps drain TMEM and run the epilogue.  16 warps up
-// to four CTAs per cluster; with more, a thread's prefetched partials need the registers of 8.  Bound:
+// to four CTAs per cluster; with more, a thread's prefetched partials need the registers of 8: n = 1152,
+// 384 steps, 8 against 16 warps, 16 starts and S = 5, 6, 8: 5.88, 5.83, 5.86 against 6.24, 6.20, 6.23 ms,
+// 64 starts 7.53, 7.48, 7.27 against 7.75, 7.64, 7.54, 128 starts and S = 6, 8 8.67, 8.50 against 9.51,
+// 8.99; n = 2500, 64 starts, S = 5, 7: 8.64, 12.14 against 8.78, 12.40.  Bound:
 // latency of the epilogue (n = 2500, 256 starts, 3 CTAs a cluster, 43 starts a CTA; cycles: setup
 // 3.1k, main loop 7.2k, wait for the accumulators 1.9k, drain 3.5k, cluster barrier 1.5k, epilogue
 // 17-22k).  A launch 22.4 us with 8 warps, 21.3 with 16, 20.1 with the halving sums.
@@ -171,9 +174,10 @@ __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint6
         : "memory");
 }
 
-// One thread of a whole warp.  The producing and issuing warps walk their loops as whole warps and
-// only the copy, MMA and commit instructions are one thread's: with the loop itself in one thread's
-// branch, every operand of those instructions had to be moved to a uniform register first.
+// One thread of a whole warp.  The producing and issuing warps walk their loops as whole warps, so that
+// the warp leaves every wait together; only the copies, MMAs and commits are one thread's.  (The loops in
+// one thread's branch take the same time: a restart batch of n = 2500, 448 steps, 256 starts 13.31 against
+// 13.30 ms, 64 starts 9.46 against 9.56 ms for 384; ragged batch of 24 instances 14.06 against 14.16 ms.)
 __device__ __forceinline__ bool elect_one()
 {
     uint32_t p;
