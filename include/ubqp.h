@@ -241,8 +241,9 @@ int ubqp_solve_batched(int32_t num, const int64_t* n, const double* const* Q,
  * aligned to its element size:
  *   Q n x n row-major (no padding), b and p n (either may be NULL = 0), x batch x n
  *   row-major, h_out batch (may be NULL), g_out batch x n (may be NULL).
- * 1 <= n <= 65536 and one point must fit in shared memory (n * element size <= 227 KiB,
- * else UBQP_ENOTSUP).  stream: cudaStream_t (NULL = default).
+ * 1 <= n <= 65536 and n * element size <= 227 KiB (else UBQP_ENOTSUP; limits of the interface), and
+ * batch * ceil(n / r) < 2^31 with r = 8, doubled up to 256 while batch * n / r exceeds eight times
+ * the SM count.  stream: cudaStream_t (NULL = default).
  * FP32 products are summed as in the inner loop's row dots (chains of four, TwoSum-compensated);
  * h is summed from pairs or in FP64.  Scratch (the row tiles' shares of h) is allocated and freed
  * on `stream` inside the call; returns after synchronizing `stream`.
@@ -272,10 +273,10 @@ int ubqp_penalized_vjp(const void* x, const void* g, const void* grad_h, int64_t
  * afford the device-wide synchronization those calls may cause.  The paper has no
  * counterpart; this is an interface variant of this library.
  *   Scratch: a static device array of UBQP_NOALLOC_SCRATCH_BYTES that every GPU loading the
- *   library holds until the process exits.  Limits: batch <= 256, n * element size <=
- *   200 KiB, and batch * ceil(n / rows per item) <= 16384 work items (rows per item as in
- *   ubqp_penalized_eval, at most 256); larger requests return UBQP_EINVAL with the limit
- *   named in ubqp_last_error().
+ *   library holds until the process exits (a call uses the first batch * ceil(n / 32) * 8 bytes,
+ *   at most 1,050,624).  Limits of the interface: batch <= 256, n * element size <= 200 KiB, and
+ *   batch * ceil(n / r) <= 16384 with r as in ubqp_penalized_eval; larger requests return
+ *   UBQP_EINVAL with the limit named in ubqp_last_error().
  *   The array's device address is resolved (cudaGetSymbolAddress) on the first call in each
  *   CUDA context, so make that first call before any stream capture in that context; a new
  *   context (after a device reset) gets its own first call.

@@ -1476,7 +1476,10 @@ class Solver {
     // each, at least one per row block, for the smallest m (tiles per CTA) at which all groups are
     // resident together.  Device time against the lane loop (three subproblems of at most 40 steps):
     // 4 lanes of n = 2000 (m = 4) 2.3 against 6.4 ms, 8 of them (m = 8) 3.5 against 6.9 ms, 4 of
-    // n = 4500 (m = 18) 7.5 against 10.4 ms; beyond kSymMaxTiles the lane loop keeps all SMs busier
+    // n = 4500 (m = 18) 7.5 against 10.4 ms, 4 of n = 4864 (m = 20) 7.8 against 10.6 ms.  kSymMaxTiles is
+    // the room of a CTA's tile table, not the crossover: with a larger table the groups stay ahead in
+    // batches of a few very unequal lanes, which alone need more (10000 and 3 x 500, m = 23, 8.0 against
+    // 14.7 ms; 14000 and 3 x 200, m = 42, 12.9 against 21.7 ms)
     bool plan_sym_groups(const std::vector<int>& ids)
     {
         auto tiles = [&](int l) { const int nb = inst_[(size_t)lane_inst_[l]].nb; return nb * (nb + 1) / 2; };
@@ -2226,8 +2229,9 @@ int ubqp_penalized_eval(const void* Q, const void* b, const void* p, const void*
     if (rc) return rc;
     cudaStream_t s = (cudaStream_t)stream;
     const size_t es = dtype == UBQP_DTYPE_F64 ? 8 : 4;
+    // (an interface limit: the kernel stages 512 bytes of a row at a time and would take longer points)
     if ((size_t)n * es > 227 * 1024) {
-        set_error("ubqp_penalized_eval: one point (n = %lld) does not fit in shared memory", (long long)n);
+        set_error("ubqp_penalized_eval: n * element size = %lld bytes exceeds the limit of 227 KiB", (long long)(n * es));
         return UBQP_ENOTSUP;
     }
     int dev = 0, sms = 148;

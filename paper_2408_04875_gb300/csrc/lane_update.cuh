@@ -142,6 +142,7 @@ __host__ __device__ __forceinline__ void sym_eig_min(float (&M)[3][3], float& la
     for (int r = 0; r < 3; ++r) v[r] = r < K ? (j == 0 ? V[r][0] : (j == 1 ? V[r][1] : V[r][2])) : 0.f;
 }
 
+// the same for a size known at run time (the host test; the kernels call rr_step, sizes 2 and 3)
 __host__ __device__ __forceinline__ void small_sym_eig_min(int k, float (&M)[3][3], float& lam, float (&v)[3])
 {
     if (k == 3) sym_eig_min<3>(M, lam, v);

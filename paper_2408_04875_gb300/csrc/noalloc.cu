@@ -2,8 +2,8 @@
 // must not allocate device memory.  Some callers manage every byte of device memory
 // through their own pool or a fixed budget and may not call cudaMalloc/cudaFree (which
 // can also synchronize the whole device); this entry point gives them the same
-// computation as ubqp_penalized_eval, with the same kernel and the same work partition,
-// with its scratch in a fixed static device array.
+// computation as ubqp_penalized_eval, with the same kernel and the same tiles, with its scratch
+// in a fixed static device array.
 //
 // The scratch (the row tiles' shares of h) lives in g_noalloc_scratch below.  Every GPU that loads
 // the library holds it until the process exits.  All calls share it and it keeps the last call's
@@ -84,7 +84,7 @@ extern "C" int ubqp_penalized_eval_noalloc(const void* Q, const void* b, const v
         return UBQP_EINVAL;
     }
     const int64_t es = dtype == UBQP_DTYPE_F64 ? 8 : 4;
-    // limits of the static scratch and of shared memory
+    // limits of the interface (they keep the shares of h within the static scratch)
     if (batch > kNoallocMaxLanes) {
         set_error("ubqp_penalized_eval_noalloc: batch = %lld exceeds the scratch limit of %d points", (long long)batch,
                   kNoallocMaxLanes);
@@ -100,7 +100,6 @@ extern "C" int ubqp_penalized_eval_noalloc(const void* Q, const void* b, const v
         set_error("ubqp_penalized_eval_noalloc: %s", cudaGetErrorString(cudaGetLastError()));
         return UBQP_ECUDA;
     }
-    // (the kernel and its partition are those of ubqp_penalized_eval, so both return the same values)
     int rb = 8;
     while (rb < 256 && batch * n / rb > 8 * (int64_t)sms) rb *= 2;
     const int64_t nblk = (n + rb - 1) / rb;
@@ -127,6 +126,7 @@ extern "C" int ubqp_penalized_eval_noalloc(const void* Q, const void* b, const v
         return UBQP_ECUDA;
     }
     cudaStream_t s = (cudaStream_t)stream;
+    // (the launch of ubqp_penalized_eval, so both return the same values)
     e = launch_grad(Q, b, p, x, n, batch, dtype, h_out, g_out, scratch, sms, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {

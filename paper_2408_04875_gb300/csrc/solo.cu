@@ -97,23 +97,19 @@ __global__ void __launch_bounds__(kThreads, 2) solo_lane_kernel(SoloArgs A)
 
     // ---- this CTA's group, its rank in the group and the group's barrier
     if (threadIdx.x == 0) {
-        int g = 0;
-        if (A.gcta) {
-            int lo = 0, hi = A.ngroups - 1;   // the last group whose first CTA is <= blockIdx.x
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (A.gcta[mid] <= (int)blockIdx.x) lo = mid;
-                else hi = mid - 1;
-            }
-            g = lo;
+        int lo = 0, hi = A.ngroups - 1;   // the last group whose first CTA is <= blockIdx.x
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (A.gcta[mid] <= (int)blockIdx.x) lo = mid;
+            else hi = mid - 1;
         }
-        s_g = g;
+        s_g = lo;
         s_ok = 1;
     }
     __syncthreads();
     const int g = s_g;
-    const int c0 = A.gcta ? A.gcta[g] : 0;
-    const int nc = A.gcta ? A.gcta[g + 1] - c0 : (int)gridDim.x;
+    const int c0 = A.gcta[g];
+    const int nc = A.gcta[g + 1] - c0;
     const int rank = (int)blockIdx.x - c0;
     unsigned long long* bar = reinterpret_cast<unsigned long long*>(A.bar + (size_t)g * kSoloBarStride);
     // barriers the group completed in earlier launches (a CTA that is already waiting at this
@@ -131,11 +127,11 @@ __global__ void __launch_bounds__(kThreads, 2) solo_lane_kernel(SoloArgs A)
     __syncthreads();
     const Params& P = sP;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int li0 = A.glanes ? A.gfirst[g] : 0, li1 = A.glanes ? A.gfirst[g + 1] : 1;
+    const int li0 = A.gfirst[g], li1 = A.gfirst[g + 1];
     int steps_left = A.budget;
 
     for (int li = li0; li < li1 && steps_left > 0; ++li) {
-        const int lane_id = A.glanes ? A.glanes[li] : 0;
+        const int lane_id = A.glanes[li];
         __syncthreads();   // shared state of the previous lane no longer in use
         if (threadIdx.x < (int)(sizeof(LaneDev) / 8))
             reinterpret_cast<int2*>(&sL)[threadIdx.x] =
@@ -286,10 +282,7 @@ __global__ void __launch_bounds__(kThreads, 2) solo_lane_kernel(SoloArgs A)
     __syncthreads();
     if (rank == 0 && threadIdx.x == 0) {
         int left = 0;
-        for (int li = li0; li < li1; ++li) {
-            const int lane_id = A.glanes ? A.glanes[li] : 0;
-            left += A.lane[lane_id].st->phase != PH_DONE ? 1 : 0;
-        }
+        for (int li = li0; li < li1; ++li) left += A.lane[A.glanes[li]].st->phase != PH_DONE ? 1 : 0;
         if (left) atomicAdd(A.active_after, left);
     }
 }

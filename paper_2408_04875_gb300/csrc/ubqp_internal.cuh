@@ -484,9 +484,9 @@ struct LoopArgs {
 // group runs its lanes one after another, every lane on all CTAs of its group
 struct SoloArgs {
     const LaneDev* lane;        // the lanes
-    const int32_t* glanes;      // lane indices, group after group (null: lane 0 alone)
+    const int32_t* glanes;      // lane indices, group after group
     const int32_t* gfirst;      // group g's lanes: glanes[gfirst[g] .. gfirst[g+1])
-    const int32_t* gcta;        // group g's CTAs: gcta[g] .. gcta[g+1]-1 (null: one group)
+    const int32_t* gcta;        // group g's CTAs: gcta[g] .. gcta[g+1]-1
     int32_t ngroups;
     int32_t rows_per_item;
     int32_t budget;             // steps each group may take in this launch
@@ -520,7 +520,7 @@ bool sell_fits(int per, bool tight, size_t smem);
 cudaError_t launch_sell(const SoloArgs& a, int per, bool tight, size_t smem, cudaStream_t s);
 
 // the same groups on the symmetric tiles, at most kSymMaxTiles tiles per CTA (sym_lane.cu)
-constexpr int kSymMaxTiles = 20;
+constexpr int kSymMaxTiles = 20;   // (plan_sym_groups says what lies beyond)
 size_t sym_lane_words(int nb);
 size_t sym_lane_smem(int ld, int tiles, int32_t* mat_bytes);
 cudaError_t launch_sym(const SoloArgs& a, size_t smem, cudaStream_t s);
