@@ -31,12 +31,11 @@ sys.path.insert(0, ROOT)
 METRIC = "inner PG iters/s (batch×n) and time-to-oracle-objective vs plain FP32 path"
 UNIT = "lane-var-updates/s"
 GEMV_KERNELS = {1: "phase_a_gemv_kernel", 2: "lane_loop_kernel"}   # 3: as the library reports it
-# DRAM bytes (read + write) per algorithmic byte of the dominant kernel, keyed by (scheduler,
-# storage), from an ncu capture of every launch of this workload's timed solve
-# (dram__bytes_read.sum + dram__bytes_write.sum over the launches against the bench's own
-# algorithmic bytes); combinations without such a capture report null (the lane-group kernels have
-# one of a capped sweep only, under profiles/)
-TRAFFIC_RATIO = {}
+# DRAM bytes (read + write) per algorithmic byte of the dominant kernel, from an ncu capture of
+# every launch of the default workload's solve (dram__bytes_read.sum + dram__bytes_write.sum over
+# the launches against the bench's own algorithmic bytes; the launch list under profiles/); other
+# kernels and workloads report null
+TRAFFIC_RATIO = {"sell_lane_kernel": 0.7922 / 37.774}
 SIZES = (250, 500, 1000, 2500)
 SEEDS_PER_SIZE = 10
 WORKLOAD = ("plain PSDP sweep: n in {250,500,1000,2500} x 10 seeded instances, density 0.1, "
@@ -663,6 +662,9 @@ def run_gpu(args):
     pa_bytes = sum(s["phase_a_bytes"] for s in stats)
     alg_bytes = sum(s["alg_bytes"] for s in stats)
     peak, peak_kind = _peaks()
+    kernel = GEMV_KERNELS.get(stats[-1]["gemv_kernel"], group_kernel)
+    whole = args.sizes == SIZES and args.seeds == SEEDS_PER_SIZE and args.max_outer is None
+    traffic = TRAFFIC_RATIO[kernel] * alg_bytes / pa_n if whole and pa_n and kernel in TRAFFIC_RATIO else None
     achieved = alg_bytes / (pa_ms * 1e-3) / 1e9 if pa_ms > 0 else None
     achieved_storage = pa_bytes / (pa_ms * 1e-3) / 1e9 if pa_ms > 0 else None
 
@@ -678,10 +680,8 @@ def run_gpu(args):
                        "ticks_per_step": stats[-1]["ticks"], "best_objectives_first3": [float(v) for v in objs[:3]]},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": (achieved / peak) if achieved else None,
-                         "traffic": (TRAFFIC_RATIO[(stats[-1]["gemv_kernel"], stats[-1]["storage"])] * alg_bytes
-                                     / max(pa_n, 1) if (stats[-1]["gemv_kernel"], stats[-1]["storage"]) in TRAFFIC_RATIO
-                                     and pa_n else None),
-                         "kernel": GEMV_KERNELS.get(stats[-1]["gemv_kernel"], group_kernel), "launches": pa_n,
+                         "traffic": traffic,
+                         "kernel": kernel, "launches": pa_n,
                          "avg_launch_us": pa_ms * 1e3 / max(pa_n, 1),
                          "algorithmic_bytes_per_launch": alg_bytes / max(pa_n, 1),
                          "algorithmic_bytes": "sparse minimum: per lane-step 6 B x stored off-diagonal entries "
@@ -695,7 +695,7 @@ def run_gpu(args):
             "gpu_launches": int(sum(s["kernel_launches"] for s in stats)),
             "clocks": clocks,
         }
-        if args.sizes != SIZES or args.seeds != SEEDS_PER_SIZE or args.max_outer is not None:
+        if not whole:
             line["config"]["workload"] = (f"profiling case: n in {list(args.sizes)} x {args.seeds} seeds, "
                                           f"max_outer={args.max_outer}")
         if not args.no_c4:
