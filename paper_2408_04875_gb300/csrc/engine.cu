@@ -1077,6 +1077,8 @@ class Solver {
                 tca.tmem_cols = tcp_tmem_cols(o_.precision == UBQP_BF16X2_TC);
                 tca.kbs = tcp_pick_kbs(max_bn_, o_.precision == UBQP_BF16X2_TC);
                 tcp_grid_ = tcp_grid(tca, tc_tiles_);
+            } else {
+                UBQP_CK(tc_prepare(tca, tc_S_));
             }
         }
         const bool timeline = o_.profile_kernels >= 2;

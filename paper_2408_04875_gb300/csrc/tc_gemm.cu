@@ -1160,8 +1160,6 @@ int tcp_grid(const TcArgs& a, int ntiles)
 cudaError_t tcp_launch(const TcArgs& a, int ntiles, int grid, cudaStream_t st)
 {
     const size_t smem = tcp_smem_bytes(a.max_bn, a.two_any != 0, a.kbs, a.stages);
-    cudaError_t e = open_smem((const void*)phase_a_tcp_kernel, smem);
-    if (e != cudaSuccess) return e;
     phase_a_tcp_kernel<<<grid, kTcpThreads, smem, st>>>(a, ntiles);
     return cudaGetLastError();
 }
@@ -1188,12 +1186,15 @@ static cudaLaunchConfig_t tc_config(int ctas, int S, size_t smem, cudaLaunchAttr
     return cfg;
 }
 
+cudaError_t tc_prepare(const TcArgs& a, int S)
+{
+    return open_smem((const void*)tc_kernel(S), tc_smem_bytes(a.max_bn, a.two_any != 0, a.stages));
+}
+
 cudaError_t tc_launch(const TcArgs& a, int total_clusters, int S, cudaStream_t st)
 {
     const size_t smem = tc_smem_bytes(a.max_bn, a.two_any != 0, a.stages);
     const TcKernel k = tc_kernel(S);
-    cudaError_t e = open_smem((const void*)k, smem);
-    if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = tc_config(total_clusters * S, S, smem, attr);
     cfg.stream = st;
@@ -1339,7 +1340,8 @@ extern "C" int ubqp_tc_matmul_probe(const uint16_t* A, const uint16_t* Bhi, cons
             le = tcp_launch(a, tiles, tcp_grid(a, tiles), nullptr);
         } else {
             const int S = cluster > 0 ? cluster : tc_pick_cluster(tiles, ld / 64, bn, two, a.stages, nsm);
-            le = tc_launch(a, tiles, S, nullptr);
+            le = tc_prepare(a, S);
+            if (le == cudaSuccess) le = tc_launch(a, tiles, S, nullptr);
         }
         if (le != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
             rc = UBQP_ECUDA;

@@ -47,8 +47,9 @@ struct TcArgs {
 
 size_t tc_smem_bytes(int bn, bool two, int stages);
 int tc_pick_stages(int bn, bool two);
+cudaError_t tc_prepare(const TcArgs& a, int S);   // once before launches of this form
 cudaError_t tc_launch(const TcArgs& a, int total_clusters, int S, cudaStream_t st);
-int tc_max_active_clusters(int bn, bool two, int stages, int S);
+int tc_max_active_clusters(int bn, bool two, int stages, int S);   // also prepares the launches
 int tc_tmem_cols(int bn, bool two);
 CUresult tc_encode_map(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, int box_rows);
 
@@ -57,7 +58,7 @@ size_t tcp_smem_bytes(int bn, bool two, int kbs, int stages);
 int tcp_pick_kbs(int bn, bool two);
 int tcp_pick_stages(int bn, bool two);   // slots of tcp_pick_kbs k-blocks
 int tcp_tmem_cols(bool two);
-int tcp_grid(const TcArgs& a, int ntiles);
+int tcp_grid(const TcArgs& a, int ntiles);        // also prepares the launches
 cudaError_t tcp_launch(const TcArgs& a, int ntiles, int grid, cudaStream_t st);
 
 // cluster size for a launch of `tiles` output tiles: the largest S <= 8 such that every
