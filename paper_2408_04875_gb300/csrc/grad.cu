@@ -16,7 +16,9 @@
 // FP32 2110 -> 970 us, i.e. 24 T FP32 operations/s of the 36 T that packed additions alone reach
 // here (two rows a thread, 16 points a CTA or FMAs in place of subtractions: no faster).
 //
-// The FP32 epilogue works in error-free pairs (TwoSum, FMA product errors) and rounds g once; FP64
+// The FP32 epilogue works in error-free pairs (TwoSum, FMA product errors) and rounds g once.  Against
+// FP64 at n = 8192, 128 points, relative root mean square (before: row products rounded to FP32, then
+// FP64): h 5.0e-8 either way, g 5.95e-8 -> 4.76e-8.  FP64
 // adds chains of eight products in two levels (four chains, then those), which keeps its rounding
 // at that of a row dot spread over 64 accumulators.
 #include <algorithm>
