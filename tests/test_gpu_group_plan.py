@@ -59,9 +59,9 @@ def test_dense_lanes(ub):
 
 # two CTAs on an SM hold two vectors of up to 12,416 entries: three lanes of 11,600 and 12,320 need more than five
 # slices per CTA with one CTA per SM, and run on the sliced kernel with two, with the bits of the lock-step
-# scheduler
-@pytest.mark.parametrize("n", [11600, 12320])
-def test_long_vectors_on_two_ctas_per_sm(ub, n):
+# scheduler; a lane of one block (20 variables) rides along
+@pytest.mark.parametrize("n,method", [(11600, 0), (12320, 0), (12320, 1)])
+def test_long_vectors_on_two_ctas_per_sm(ub, n, method):
     import torch
     Qs = []
     for k in range(3):
@@ -71,7 +71,9 @@ def test_long_vectors_on_two_ctas_per_sm(ub, n):
         u = torch.triu(v)
         Qs.append((u + torch.triu(v, 1).T).contiguous())
         del v, u
-    kw = dict(max_outer=2, max_inner=30, seed=1)
+    Qs.append(Qs[0][:20, :20] + 7 * torch.eye(20, device="cuda", dtype=torch.float64))
+    Qs[-1][3, 11] = Qs[-1][11, 3] = -40
+    kw = dict(max_outer=2, max_inner=30, seed=1, method=method)
     xs, f, st = ub.solve_batched(Qs, None, lane_budget=40, **kw)
     g = ub.lane_groups()
     assert st["gemv_kernel"] == 3
